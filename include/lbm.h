@@ -182,9 +182,10 @@ lbm_status lbm_get_splitting(const lbm_sim *sim, int *scheme);
 lbm_status lbm_set_transport(lbm_sim *sim, int order);
 lbm_status lbm_get_transport(const lbm_sim *sim, int *order);
 
-/* Kernel variant: the number of warps that share one 32-cell segment (1, 2, 3, 4 or 6
- * dividing M; each warp owns M/warps velocity rows), and the load path of the wall-free
- * segments: 0 registers, 1 registers with all loads issued ahead of the arithmetic,
+/* Kernel variant: the number of velocity slices of a cell -- on load paths 2 and up the warps
+ * that share one 32-cell segment -- (1, 2, 3, 4 or 6 dividing M; each owns M/slices velocity
+ * rows), and the load path: 0 and 1 registers (one kernel for all cells; the block's cells
+ * follow from the slices, and until a variant is set the library picks both by the grid),
  * 2 TMA (bulk asynchronous copies into shared memory, FP32 cavities with nx and the cell
  * count multiples of 4 and the planar state layout; M = 8 or 12), 3 as 2 with the wall
  * segments in the same launch,

@@ -4,7 +4,7 @@
 // block of time steps, captured once into a CUDA graph and replayed.
 //
 // Each time step is the paper's fully discrete scheme (Eqs. 1, 5-9; the same arithmetic
-// as step_kernel.cuh) applied to every active instance.  Work items are (instance,
+// as step_tile.cuh) applied to every active instance.  Work items are (instance,
 // 32-cell segment) pairs in a schedule order chosen by the autotuner; the blocks of the
 // persistent grid take items round-robin, a grid-wide barrier separates time steps, and
 // every `resid_every` steps the per-instance residuals are reduced (FP64 atomics) and
@@ -32,7 +32,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_internal.h"
-#include "step_kernel.cuh"
+#include "step_wall.cuh"
 
 lbm_status lbm_norms_fail(lbm_status s, const char *msg);
 

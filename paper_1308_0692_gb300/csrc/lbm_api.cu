@@ -17,11 +17,12 @@
 #include "../../include/lbm.h"
 #include "lbm_internal.h"
 
-cudaError_t launch_step_f64_small(int m, int g, int pf, bool resid, const StepArgs &a, int grid, cudaStream_t s);
-cudaError_t launch_step_f64_large(int m, int g, int pf, bool resid, const StepArgs &a, int grid, cudaStream_t s);
-cudaError_t launch_step_f32_small(int m, int g, int pf, bool resid, const StepArgs &a, int grid, cudaStream_t s);
-cudaError_t launch_step_f32_large(int m, int g, int pf, bool resid, const StepArgs &a, int grid, cudaStream_t s);
-cudaError_t launch_defect_f32(int m, const StepArgs &a, int grid, cudaStream_t s);
+cudaError_t launch_step_f64_small(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s);
+cudaError_t launch_step_f64_large(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s);
+cudaError_t launch_step_f32_small(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s);
+cudaError_t launch_step_f32_large(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s);
+cudaError_t launch_defect_f32(int m, int ns, const StepArgs &a, cudaStream_t s);
+cudaError_t launch_correct_f32(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s);
 cudaError_t launch_step_f32_tma(int m, int g, bool resid, const StepArgs &a, int grid, cudaStream_t s,
                                bool merged);
 cudaError_t prepare_step_f32_tma(int m, int g);
@@ -39,11 +40,6 @@ bool so_march_supported(int m, int g, int slots, int tiled);
 static int so_march_slots(int pf) { return pf == 8 ? 5 : 4; }
 static int so_march_tiled(int pf) { return pf == 8 ? 1 : 2; }
 bool march_supported(int m, int g, int slots, bool defer, int tiled);
-int defect_lanes(int m);
-int correct_lanes(int m);
-cudaError_t launch_correct_f32(int m, int g, bool resid, const StepArgs &a, int grid,
-                               cudaStream_t s);
-
 struct lbm_vset {
     int kind;
     int n_arg;
@@ -59,7 +55,9 @@ struct lbm_sim {
     long ncells;
     double dt, dx, dy, omega, u_ref;
     cudaStream_t stream;
-    int lanes;            // warps per 32-cell segment of the step kernel
+    int lanes;            // warps per 32-cell segment of the step kernel (load paths 0, 1: velocity slices)
+    bool lanes_set;       // lanes chosen by lbm_set_variant; else tile_plan picks the slices of load path 0
+    int slices;           // velocity slices of load paths 0 and 1
     int prefetch;         // load path of the wall-free cells (lbm_set_variant)
     int splitting;        // LBM_SPLIT_LIE (stored state h) or LBM_SPLIT_STRANG[_EXACT] (stored g = R(dt/2) h)
     int order;            // transport order: 1 (first-order upwind, the paper's) or 2
@@ -168,9 +166,9 @@ Layout make_layout(const lbm_vset *vs, const lbm_problem *p)
     L.wall_cap = 2 * (p->nx + p->ny) + 4;
     L.off_wsegs = off;
     off = align256(off + sizeof(int) * L.wall_cap);
-    // the finest bulk launch has one 32-cell segment per block, plus the wall kernel's
-    // blocks; norms use at most 152*8 blocks
-    long nb = (ncells + 31) / 32 + L.wall_cap;
+    // the finest launch has four cells a block (tile_plan) or, on the segment paths, 32-cell
+    // segments and the wall kernel's blocks; norms use at most 152*8 blocks
+    long nb = std::max((ncells + 3) / 4 + 8L * p->nx, (ncells + 31) / 32 + L.wall_cap);
     if (nb < 152 * 8) nb = 152 * 8;
     L.npartials = (int)nb;
     L.off_partials = off;
@@ -364,6 +362,7 @@ void fill_args(lbm_sim *s, const TableHeader &hdr)
         a.nux[i] = column ? 0.0 : std::fabs(v.nodes[i]) * s->dt / s->dx;
         a.nuy[i] = std::fabs(v.nodes[i]) * s->dt / s->dy;
         a.w1[i] = v.weights[i];
+        a.wxi[i] = a.w1[i] * a.xi[i];
         a.xi_f[i] = (float)a.xi[i];
         a.nux_f[i] = (float)a.nux[i];
         a.nuy_f[i] = (float)a.nuy[i];
@@ -378,6 +377,8 @@ void fill_args(lbm_sim *s, const TableHeader &hdr)
             a.so_c_f[ax][i] = (float)a.so_c[ax][i];
         }
     }
+    for (int iy = 0; iy < v.m; ++iy)
+        for (int ix = 0; ix < v.m; ++ix) a.a0[iy * v.m + ix] = 1.0 - a.nux[ix] - a.nuy[iy];
     a.omega = s->omega;
     a.b = 1.0 - s->omega;
     a.omega_f = (float)a.omega;
@@ -388,6 +389,40 @@ void fill_args(lbm_sim *s, const TableHeader &hdr)
     a.u_top = p.u_top;
     a.inv_u_ref = 1.0 / s->u_ref;
 }
+
+// Velocity slices and cells of a block of step_tile.cuh (load paths 0 and 1, the correction
+// march; dp: FP64 arithmetic, the FP64 march and the defect pass).  Measured over 19 grids
+// (1 x 100 to 512 x 512, M = 3 to 12; us per step, replayed graphs):
+//   FP64 is bound by the FP64 pipe of each SM quarter, so small blocks that spread evenly win,
+//     with one velocity row a thread while the grid leaves the quarters short of warps (M = 8:
+//     64^2 12.1 against 15.6 with two rows, 128^2 25.2 against 28.1) and two or three rows a
+//     thread beyond (M = 8: 192^2 48.1 against 50.0; M = 12: 128^2 51.9 against 54.4, 300^2
+//     223.5 against 225.2, 512^2 614 against 624);
+//   FP32 is bound by the L2's latency and traffic: 16 places with two rows a thread (M = 8:
+//     128^2 4.8; 32 places 5.9, one row a thread 6.0), 32 places where there are enough of
+//     them to fill the chip (333 x 251 10.4 against 10.8), few cells with one row a thread
+//     (40 x 33 2.9 against 3.2); small sets whole rows a thread (M = 4: 128^2 2.7 against 2.9).
+struct TilePlan {
+    int ns, w, r;
+};
+
+TilePlan tile_plan(bool dp, int m, long ncells)
+{
+    if (m == 3) return {1, 16, 2};
+    if (dp) {
+        if (m == 4) return {4, 8, 1};
+        if (m == 6) return {6, 8, 2};
+        if (m == 8) return ncells < 25000 ? TilePlan{8, 4, 1} : TilePlan{4, 8, 1};
+        return ncells < 100000 ? TilePlan{12, 8, 1} : TilePlan{4, 8, 1};
+    }
+    if (m == 4) return ncells < 4000 ? TilePlan{4, 16, 2} : ncells < 50000 ? TilePlan{1, 16, 2} : TilePlan{1, 32, 2};
+    if (m == 6) return ncells < 20000 ? TilePlan{6, 8, 2} : TilePlan{2, 32, 1};
+    if (m == 8) return ncells < 2500 ? TilePlan{8, 8, 1} : ncells < 50000 ? TilePlan{4, 16, 1} : TilePlan{4, 32, 1};
+    return {6, 16, 1};
+}
+
+// the same for slices the caller chose (lbm_set_variant)
+TilePlan tile_plan_for(bool dp, int ns) { return dp ? TilePlan{ns, 8, ns == 1 ? 4 : 1} : TilePlan{ns, ns >= 6 ? 16 : 32, ns == 1 ? 2 : 1}; }
 
 int grid_for(long ncells, int lanes)
 {
@@ -420,7 +455,7 @@ cudaError_t enqueue_steps(lbm_sim *s, long first, long count, int cur, cudaStrea
                                                             so_march_tiled(s->prefetch), resid, a, s->grid, st)
                                  : launch_step_so(s->prob.prec, s->vs.m, s->lanes, resid, a, s->grid, st);
         else
-            e = launch_step(s->prob.prec, s->vs.m, s->lanes, s->prefetch, resid, a, s->grid, st);
+            e = launch_step(s->prob.prec, s->vs.m, s->prefetch <= 1 ? s->slices : s->lanes, s->prefetch, resid, a, s->grid, st);
         if (e != cudaSuccess) return e;
         if (resid) {
             e = launch_finalize_residual(s->partials, s->nparts_step, s->result, st);
@@ -499,9 +534,6 @@ lbm_status set_lanes(lbm_sim *s, int lanes)
     s->grid = grid_for(s->ncells, lanes);
     s->args.wall_segs = s->wall_segs;
     s->args.n_wall_segs = (int)segs.size();
-    // one merged launch when wall segments are more than a tenth of all segments
-    const long nseg_total = (s->ncells + 31) / 32;
-    s->args.merged = (long)segs.size() * 10 > nseg_total ? 1 : 0;
     if (s->prefetch >= 4) {
         int strips = 0, chunks = 0;
         // every march block writes one residual partial: the march grid and the wall kernel's
@@ -515,9 +547,16 @@ lbm_status set_lanes(lbm_sim *s, int lanes)
         s->args.march_strips = strips;
         s->args.march_chunks = chunks;
         s->args.counters = (int *)(s->result + 12);
-        s->args.merged = 0;
     }
     s->nparts_step = s->grid + wall_grid(lanes, (int)segs.size());
+    if (s->order == 1 && s->prefetch <= 1) {
+        const bool dp = s->prob.prec == LBM_FP64;
+        const TilePlan t = s->lanes_set ? tile_plan_for(dp, lanes) : tile_plan(dp, s->vs.m, s->ncells);
+        s->slices = t.ns;
+        s->args.tile_w = t.w;
+        s->args.tile_r = t.r;
+        s->nparts_step = s->grid = (int)tile_blocks(nx, ny, t.w, t.r);
+    }
     if (s->nparts_step > s->npartials) return fail(LBM_EINVAL, "internal: residual partials overflow");
     return LBM_OK;
 }
@@ -564,10 +603,8 @@ cudaError_t launch_step(int prec, int m, int g, int pf, bool resid, const StepAr
     if (pf >= 4 && pf <= 9)
         return launch_step_f32_march(m, g, march_slots(pf), march_defer(pf), march_tiled(pf), resid, a, grid, s);
     if (prec == LBM_FP64)
-        return m >= 8 ? launch_step_f64_large(m, g, pf, resid, a, grid, s)
-                      : launch_step_f64_small(m, g, pf, resid, a, grid, s);
-    return m >= 12 ? launch_step_f32_large(m, g, pf, resid, a, grid, s)
-                   : launch_step_f32_small(m, g, pf, resid, a, grid, s);
+        return m >= 8 ? launch_step_f64_large(m, g, resid, a, s) : launch_step_f64_small(m, g, resid, a, s);
+    return m >= 12 ? launch_step_f32_large(m, g, resid, a, s) : launch_step_f32_small(m, g, resid, a, s);
 }
 
 extern "C" {
@@ -696,6 +733,7 @@ lbm_status lbm_init(const lbm_vset *vs, const lbm_problem *prob, const double *i
     s->ncells = (long)prob->nx * prob->ny;
     s->stream = (cudaStream_t)stream;
     s->lanes = default_lanes_per_cell(prob->prec, vs->m);
+    s->lanes_set = false;
     s->prefetch = 0;
     s->splitting = LBM_SPLIT_LIE;
     s->order = 1;
@@ -846,20 +884,18 @@ lbm_status read_result(lbm_sim *s, double out[4])
     return LBM_OK;
 }
 
-int nparts_for(const lbm_sim *s, int lanes)
-{
-    return grid_for(s->ncells, lanes) + wall_grid(lanes, s->args.n_wall_segs);
-}
-
 // FP64 defect of the FP32 state H: D = M64(H) - H (float); returns ||D||^2, ||M64(H)||^2.
 lbm_status defect_pass(lbm_sim *s, void *H, void *D, double *dsum, double *nsum)
 {
     StepArgs a = s->args;
     a.h = H;
     a.hn = D;
-    const int g = defect_lanes(s->vs.m);
-    cudaError_t e = launch_defect_f32(s->vs.m, a, grid_for(s->ncells, g), s->stream);
-    if (e == cudaSuccess) e = launch_finalize_residual(s->partials, nparts_for(s, g), s->result, s->stream);
+    const TilePlan t = tile_plan(true, s->vs.m, s->ncells);
+    a.tile_w = t.w;
+    a.tile_r = t.r;
+    cudaError_t e = launch_defect_f32(s->vs.m, t.ns, a, s->stream);
+    if (e == cudaSuccess)
+        e = launch_finalize_residual(s->partials, (int)tile_blocks(a.nx, a.ny, t.w, t.r), s->result, s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "launching the defect pass");
     double r[4];
     lbm_status st = read_result(s, r);
@@ -927,8 +963,8 @@ lbm_status lbm_solve(lbm_sim *s, double tol, long max_steps, int refine_sweeps, 
         if (st != LBM_OK) return st;
         double r64 = nsum > 0 ? std::sqrt(dsum / nsum) : 0.0;
         const double hnorm = std::sqrt(nsum);
-        const int g = correct_lanes(s->vs.m);
-        const int grid = grid_for(s->ncells, g), nparts = nparts_for(s, g);
+        const TilePlan t = tile_plan(false, s->vs.m, s->ncells);
+        const int nparts = (int)tile_blocks(s->prob.nx, s->prob.ny, t.w, t.r);
         const double ctol = refine_tol > 0 ? refine_tol : 0.1 * tol;
         const size_t state_bytes = (size_t)s->nv * s->ncells * sizeof(float);
         // sweeps until the FP64 defect -- the FP64 march's own residual, evaluated on the
@@ -942,6 +978,8 @@ lbm_status lbm_solve(lbm_sim *s, double tol, long max_steps, int refine_sweeps, 
             StepArgs a = s->args;
             a.src = D;
             a.homogeneous = 1;
+            a.tile_w = t.w;
+            a.tile_r = t.r;
             // one interval of K correction steps (+ the residual finalisation) from C[p]
             auto enqueue_interval = [&](int p, cudaStream_t st) -> cudaError_t {
                 int q = p;
@@ -949,7 +987,7 @@ lbm_status lbm_solve(lbm_sim *s, double tol, long max_steps, int refine_sweeps, 
                     StepArgs b = a;
                     b.h = C[q];
                     b.hn = C[q ^ 1];
-                    cudaError_t err = launch_correct_f32(s->vs.m, g, j == K, b, grid, st);
+                    cudaError_t err = launch_correct_f32(s->vs.m, t.ns, j == K, b, st);
                     if (err == cudaSuccess && j == K)
                         err = launch_finalize_residual(s->partials, nparts, s->result, st);
                     if (err != cudaSuccess) return err;
@@ -1081,6 +1119,7 @@ static lbm_status set_variant_order2(lbm_sim *s, int warps_per_segment, int pref
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "changing the state layout");
     s->prefetch = prefetch;
+    s->lanes_set = true;
     return set_lanes(s, warps_per_segment);
 }
 
@@ -1117,6 +1156,7 @@ lbm_status lbm_set_variant(lbm_sim *s, int warps_per_segment, int prefetch)
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "changing the state layout");
     s->prefetch = prefetch;
+    s->lanes_set = true;
     return set_lanes(s, warps_per_segment);
 }
 
@@ -1149,6 +1189,7 @@ lbm_status lbm_set_transport(lbm_sim *s, int order)
     if (s->step != 0) return fail(LBM_EINVAL, "the transport order is chosen before the first step");
     s->order = order;
     s->prefetch = 0;
+    s->lanes_set = false;
     cudaError_t e = set_tiled(s, false);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "changing the state layout");

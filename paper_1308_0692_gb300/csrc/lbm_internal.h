@@ -69,8 +69,7 @@ struct StepArgs {
     int n_wall_segs;
     long partials_offset; // first partials slot of the wall kernel
     int *status;          // set to 1 by a device-side wait that gave up
-    int merged;           // bulk and wall segments in one launch
-    int bulk_blocks;      // merged launch: blocks taking the wall-free segments
+    int tile_w, tile_r;   // step_tile.cuh: places and rows of a block's cells
     int wall_blocks;      // merged TMA launch: leading blocks taking the wall segments
     int *counters;        // column march: [0] next item, [1] finished blocks (zero between launches)
     int march_strips;     // column march: 64-cell strips of the interior
@@ -80,6 +79,8 @@ struct StepArgs {
     double nux[LBM_MAX_M];  // |xi| dt / dx (0 for a single periodic Couette column)
     double nuy[LBM_MAX_M];  // |xi| dt / dy
     double w1[LBM_MAX_M];   // 1-D weights (w_a = w1[ix] w1[iy])
+    double wxi[LBM_MAX_M];  // w1 xi
+    double a0[LBM_MAX_V];   // 1 - nux[ix] - nuy[iy]
     float xi_f[LBM_MAX_M], nux_f[LBM_MAX_M], nuy_f[LBM_MAX_M], w1_f[LBM_MAX_M];
     // second-order transport, per axis (0: x, 1: y) and node with Courant number nu:
     // P = nu (3 - nu) / 2, B = nu (2 - nu), and the second upwind cell's coefficient
@@ -94,12 +95,15 @@ struct StepArgs {
     double inv_u_ref;       // 1 / u_ref
 };
 
-// Launchers (step_*.cu).  `g` selects the warps per 32-cell segment; a launch is the
-// bulk kernel over `grid` blocks followed by the wall kernel over the wall segments; the
-// residual partials of one step occupy grid + wall_grid(g, n_wall_segs) slots.
+// Blocks of step_tile.cuh over an nx x ny grid with W places of R rows a block.
+inline long tile_blocks(int nx, int ny, int W, int R) { return ((long)nx * ((ny + R - 1) / R) + W - 1) / W; }
+
+// Launchers (step_*.cu).  Load paths 0 and 1 (step_tile.cuh): one launch over tile_blocks
+// blocks, `g` velocity slices.  The others: `g` warps per 32-cell segment, the interior kernel
+// over `grid` blocks with the wall kernel over the wall segments, whose residual partials
+// occupy grid + wall_grid(g, n_wall_segs) slots.
 cudaError_t launch_step(int prec, int m, int g, int pf, bool resid, const StepArgs &a, int grid,
                         cudaStream_t s);
-cudaError_t launch_defect(int m, const StepArgs &a, int grid, cudaStream_t s);
 int default_lanes_per_cell(int prec, int m);
 inline int segs_per_block(int g) { return g >= 8 ? 1 : 8 / g; }
 inline int wall_grid(int g, int n_wall_segs) { return (n_wall_segs + segs_per_block(g) - 1) / segs_per_block(g); }

@@ -3,40 +3,29 @@
 //             change M(h) - h (the defect) as float, with its norms;
 //   correct : the FP32 step of the homogeneous problem (wall driving removed) plus a
 //             source array -- the correction equation delta = L(delta) + defect.
-// (generated instantiation list; the kernel is in step_kernel.cuh)
-#include "step_kernel.cuh"
+// The slices are those tile_plan (lbm_api.cu) picks for either arithmetic.
+// (instantiation list; the kernel is in step_tile.cuh)
+#include "step_tile.cuh"
 
 using namespace lbmk;
 
-cudaError_t launch_defect_f32(int m, const StepArgs &a, int grid, cudaStream_t s)
+cudaError_t launch_defect_f32(int m, int ns, const StepArgs &a, cudaStream_t s)
 {
-    if (m == 3) return launch_one<float, double, 3, 1, false, false, true>(a, grid, s);
-    if (m == 4) return launch_one<float, double, 4, 1, false, false, true>(a, grid, s);
-    if (m == 6) return launch_one<float, double, 6, 2, false, false, true>(a, grid, s);
-    if (m == 8) return launch_one<float, double, 8, 4, false, false, true>(a, grid, s);
-    if (m == 12) return launch_one<float, double, 12, 6, false, false, true>(a, grid, s);
+#define LBM_DEFECT(M_, NS_) \
+    if (m == M_ && ns == NS_) return launch_tile<float, double, M_, NS_, false, false, true>(a, s);
+    LBM_DEFECT(3, 1) LBM_DEFECT(4, 4) LBM_DEFECT(6, 6) LBM_DEFECT(8, 4) LBM_DEFECT(8, 8) LBM_DEFECT(12, 4) LBM_DEFECT(12, 12)
+#undef LBM_DEFECT
     return cudaErrorInvalidValue;
 }
 
-int defect_lanes(int m) { return m == 12 ? 6 : m == 8 ? 4 : m == 6 ? 2 : 1; }
-int correct_lanes(int m) { return m == 12 ? 4 : m == 8 ? 2 : 1; }
-
-cudaError_t launch_correct_f32(int m, int g, bool resid, const StepArgs &a, int grid, cudaStream_t s)
+cudaError_t launch_correct_f32(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s)
 {
-    if (m == 3 && g == 1)
-        return resid ? launch_one<float, float, 3, 1, true, true, false>(a, grid, s)
-                     : launch_one<float, float, 3, 1, false, true, false>(a, grid, s);
-    if (m == 4 && g == 1)
-        return resid ? launch_one<float, float, 4, 1, true, true, false>(a, grid, s)
-                     : launch_one<float, float, 4, 1, false, true, false>(a, grid, s);
-    if (m == 6 && g == 1)
-        return resid ? launch_one<float, float, 6, 1, true, true, false>(a, grid, s)
-                     : launch_one<float, float, 6, 1, false, true, false>(a, grid, s);
-    if (m == 8 && g == 2)
-        return resid ? launch_one<float, float, 8, 2, true, true, false>(a, grid, s)
-                     : launch_one<float, float, 8, 2, false, true, false>(a, grid, s);
-    if (m == 12 && g == 4)
-        return resid ? launch_one<float, float, 12, 4, true, true, false>(a, grid, s)
-                     : launch_one<float, float, 12, 4, false, true, false>(a, grid, s);
+#define LBM_CORRECT(M_, NS_)                                                                       \
+    if (m == M_ && ns == NS_)                                                                      \
+        return resid ? launch_tile<float, float, M_, NS_, true, true, false>(a, s)                 \
+                     : launch_tile<float, float, M_, NS_, false, true, false>(a, s);
+    LBM_CORRECT(3, 1) LBM_CORRECT(4, 1) LBM_CORRECT(4, 4) LBM_CORRECT(6, 2) LBM_CORRECT(6, 6) LBM_CORRECT(8, 4) LBM_CORRECT(8, 8)
+    LBM_CORRECT(12, 6)
+#undef LBM_CORRECT
     return cudaErrorInvalidValue;
 }

@@ -1,38 +1,18 @@
-// FP32 fused step, 3/4/6/8 nodes per axis (perturbation stored and marched in float;
-// wall sums across velocity rows and residual reductions across threads in double).
-// (instantiation list; the kernel is in step_kernel.cuh)
-#include "step_kernel.cuh"
+// FP32 fused step, 3/4/6/8 nodes per axis (storage and arithmetic in float): velocity slices NS per nodes M an axis.
+// (instantiation list; the kernel is in step_tile.cuh)
+#include "step_tile.cuh"
 
 using namespace lbmk;
 
-cudaError_t launch_step_f32_small(int m, int g, int pf, bool resid, const StepArgs &a, int grid, cudaStream_t s)
+#define LBM_TILE_LIST(X) X(3, 1) X(4, 1) X(4, 4) X(6, 1) X(6, 2) X(6, 6) X(8, 1) X(8, 2) X(8, 4) X(8, 8)
+
+cudaError_t launch_step_f32_small(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s)
 {
-    if (m == 3 && g == 1 && pf == 0)
-        return resid ? launch_one<float, float, 3, 1, true, false, false, false>(a, grid, s)
-                     : launch_one<float, float, 3, 1, false, false, false, false>(a, grid, s);
-    if (m == 4 && g == 1 && pf == 0)
-        return resid ? launch_one<float, float, 4, 1, true, false, false, false>(a, grid, s)
-                     : launch_one<float, float, 4, 1, false, false, false, false>(a, grid, s);
-    if (m == 6 && g == 1 && pf == 0)
-        return resid ? launch_one<float, float, 6, 1, true, false, false, false>(a, grid, s)
-                     : launch_one<float, float, 6, 1, false, false, false, false>(a, grid, s);
-    if (m == 6 && g == 2 && pf == 0)
-        return resid ? launch_one<float, float, 6, 2, true, false, false, false>(a, grid, s)
-                     : launch_one<float, float, 6, 2, false, false, false, false>(a, grid, s);
-    if (m == 8 && g == 1 && pf == 0)
-        return resid ? launch_one<float, float, 8, 1, true, false, false, false>(a, grid, s)
-                     : launch_one<float, float, 8, 1, false, false, false, false>(a, grid, s);
-    if (m == 8 && g == 2 && pf == 0)
-        return resid ? launch_one<float, float, 8, 2, true, false, false, false>(a, grid, s)
-                     : launch_one<float, float, 8, 2, false, false, false, false>(a, grid, s);
-    if (m == 8 && g == 4 && pf == 0)
-        return resid ? launch_one<float, float, 8, 4, true, false, false, false>(a, grid, s)
-                     : launch_one<float, float, 8, 4, false, false, false, false>(a, grid, s);
-    if (m == 8 && g == 2 && pf == 1)
-        return resid ? launch_one<float, float, 8, 2, true, false, false, true>(a, grid, s)
-                     : launch_one<float, float, 8, 2, false, false, false, true>(a, grid, s);
-    if (m == 8 && g == 4 && pf == 1)
-        return resid ? launch_one<float, float, 8, 4, true, false, false, true>(a, grid, s)
-                     : launch_one<float, float, 8, 4, false, false, false, true>(a, grid, s);
+#define LBM_TILE_LAUNCH(M_, NS_)                                                                   \
+    if (m == M_ && ns == NS_)                                                                      \
+        return resid ? launch_tile<float, float, M_, NS_, true, false, false>(a, s)              \
+                     : launch_tile<float, float, M_, NS_, false, false, false>(a, s);
+    LBM_TILE_LIST(LBM_TILE_LAUNCH)
+#undef LBM_TILE_LAUNCH
     return cudaErrorInvalidValue;
 }

@@ -1,31 +1,18 @@
-// FP64 fused step, 8/12 nodes per axis (storage and arithmetic in double).
-// (instantiation list; the kernel is in step_kernel.cuh)
-#include "step_kernel.cuh"
+// FP64 fused step, 8/12 nodes per axis (storage and arithmetic in double): velocity slices NS per nodes M an axis.
+// (instantiation list; the kernel is in step_tile.cuh)
+#include "step_tile.cuh"
 
 using namespace lbmk;
 
-cudaError_t launch_step_f64_large(int m, int g, int pf, bool resid, const StepArgs &a, int grid, cudaStream_t s)
+#define LBM_TILE_LIST(X) X(8, 2) X(8, 4) X(8, 8) X(12, 3) X(12, 4) X(12, 6) X(12, 12)
+
+cudaError_t launch_step_f64_large(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s)
 {
-    if (m == 8 && g == 2 && pf == 0)
-        return resid ? launch_one<double, double, 8, 2, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 8, 2, false, false, false, false>(a, grid, s);
-    if (m == 8 && g == 4 && pf == 0)
-        return resid ? launch_one<double, double, 8, 4, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 8, 4, false, false, false, false>(a, grid, s);
-    if (m == 12 && g == 3 && pf == 0)
-        return resid ? launch_one<double, double, 12, 3, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 12, 3, false, false, false, false>(a, grid, s);
-    if (m == 12 && g == 4 && pf == 0)
-        return resid ? launch_one<double, double, 12, 4, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 12, 4, false, false, false, false>(a, grid, s);
-    if (m == 12 && g == 6 && pf == 0)
-        return resid ? launch_one<double, double, 12, 6, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 12, 6, false, false, false, false>(a, grid, s);
-    if (m == 8 && g == 4 && pf == 1)
-        return resid ? launch_one<double, double, 8, 4, true, false, false, true>(a, grid, s)
-                     : launch_one<double, double, 8, 4, false, false, false, true>(a, grid, s);
-    if (m == 12 && g == 6 && pf == 1)
-        return resid ? launch_one<double, double, 12, 6, true, false, false, true>(a, grid, s)
-                     : launch_one<double, double, 12, 6, false, false, false, true>(a, grid, s);
+#define LBM_TILE_LAUNCH(M_, NS_)                                                                   \
+    if (m == M_ && ns == NS_)                                                                      \
+        return resid ? launch_tile<double, double, M_, NS_, true, false, false>(a, s)              \
+                     : launch_tile<double, double, M_, NS_, false, false, false>(a, s);
+    LBM_TILE_LIST(LBM_TILE_LAUNCH)
+#undef LBM_TILE_LAUNCH
     return cudaErrorInvalidValue;
 }

@@ -1,31 +1,18 @@
-// FP64 fused step, 3/4/6 nodes per axis (storage and arithmetic in double).
-// (instantiation list; the kernel is in step_kernel.cuh)
-#include "step_kernel.cuh"
+// FP64 fused step, 3/4/6 nodes per axis (storage and arithmetic in double): velocity slices NS per nodes M an axis.
+// (instantiation list; the kernel is in step_tile.cuh)
+#include "step_tile.cuh"
 
 using namespace lbmk;
 
-cudaError_t launch_step_f64_small(int m, int g, int pf, bool resid, const StepArgs &a, int grid, cudaStream_t s)
+#define LBM_TILE_LIST(X) X(3, 1) X(4, 1) X(4, 2) X(4, 4) X(6, 1) X(6, 2) X(6, 6)
+
+cudaError_t launch_step_f64_small(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s)
 {
-    if (m == 3 && g == 1 && pf == 0)
-        return resid ? launch_one<double, double, 3, 1, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 3, 1, false, false, false, false>(a, grid, s);
-    if (m == 4 && g == 1 && pf == 0)
-        return resid ? launch_one<double, double, 4, 1, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 4, 1, false, false, false, false>(a, grid, s);
-    if (m == 4 && g == 2 && pf == 0)
-        return resid ? launch_one<double, double, 4, 2, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 4, 2, false, false, false, false>(a, grid, s);
-    if (m == 6 && g == 1 && pf == 0)
-        return resid ? launch_one<double, double, 6, 1, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 6, 1, false, false, false, false>(a, grid, s);
-    if (m == 6 && g == 2 && pf == 0)
-        return resid ? launch_one<double, double, 6, 2, true, false, false, false>(a, grid, s)
-                     : launch_one<double, double, 6, 2, false, false, false, false>(a, grid, s);
-    if (m == 4 && g == 2 && pf == 1)
-        return resid ? launch_one<double, double, 4, 2, true, false, false, true>(a, grid, s)
-                     : launch_one<double, double, 4, 2, false, false, false, true>(a, grid, s);
-    if (m == 6 && g == 2 && pf == 1)
-        return resid ? launch_one<double, double, 6, 2, true, false, false, true>(a, grid, s)
-                     : launch_one<double, double, 6, 2, false, false, false, true>(a, grid, s);
+#define LBM_TILE_LAUNCH(M_, NS_)                                                                   \
+    if (m == M_ && ns == NS_)                                                                      \
+        return resid ? launch_tile<double, double, M_, NS_, true, false, false>(a, s)              \
+                     : launch_tile<double, double, M_, NS_, false, false, false>(a, s);
+    LBM_TILE_LIST(LBM_TILE_LAUNCH)
+#undef LBM_TILE_LAUNCH
     return cudaErrorInvalidValue;
 }

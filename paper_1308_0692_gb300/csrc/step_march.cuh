@@ -1,6 +1,6 @@
 // Interior of the FP32 step as a column march with TMA staging (sm_103a).
 //
-// The same update as the bulk path of step_kernel.cuh (first-order upwind transport, then
+// The same update as the planar kernel of step_tile.cuh (first-order upwind transport, then
 // relaxation towards w_a (rho' + xi_a . j'), Eqs. 5-7 with the scheme's discretisation),
 // organised so that every value of the old state crosses the L2 -> SM path about once:
 //
@@ -644,7 +644,7 @@ cudaError_t prepare_march(int *grid)
 template <int M, int G, bool RESID, int TILED = 0>
 __global__ void __launch_bounds__(Shape<G>::THREADS) step_wall_beside_march_kernel(const StepArgs a)
 {
-    step_body<float, float, M, G, RESID, false, false, true, false, TILED != 0>(a, blockIdx.x);
+    wall_body<M, G, RESID, TILED != 0>(a, blockIdx.x);
     if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 

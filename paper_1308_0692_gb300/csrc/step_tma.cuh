@@ -1,5 +1,5 @@
 // Bulk (wall-free) segments of the fused step with TMA staging of the upwind halo
-// (sm_103a): the same arithmetic as the bulk path of step_kernel.cuh, but every warp first
+// (sm_103a): the same arithmetic as the planar kernel of step_tile.cuh, but every warp first
 // has the Tensor Memory Accelerator copy, with 1-D bulk asynchronous copies
 // (cp.async.bulk ... mbarrier::complete_tx), all the data its velocity rows need into
 // shared memory: per velocity the own-cell line widened by 4 cells on each side (the x
@@ -18,7 +18,7 @@
 
 #include <cstdint>
 
-#include "step_kernel.cuh"
+#include "step_wall.cuh"
 
 namespace lbmk {
 
@@ -274,7 +274,7 @@ template <int M, int G, bool RESID>
 __global__ void __launch_bounds__(Shape<G>::THREADS) step_tma_merged_kernel(const StepArgs a)
 {
     if ((int)blockIdx.x < a.wall_blocks)
-        step_body<float, float, M, G, RESID, false, false, true, false>(a, blockIdx.x);
+        wall_body<M, G, RESID, false>(a, blockIdx.x);
     else
         tma_body<M, G, RESID>(a, blockIdx.x - a.wall_blocks);
 }
@@ -314,7 +314,7 @@ cudaError_t launch_tma(const StepArgs &a, int grid, cudaStream_t s, bool merged)
     StepArgs b = a;
     b.partials_offset = grid;
     const int wgrid = (a.n_wall_segs + Shape<G>::SPB - 1) / Shape<G>::SPB;
-    step_kernel<float, float, M, G, RESID, false, false, true, false><<<wgrid, T, 0, s>>>(b);
+    wall_kernel<M, G, RESID><<<wgrid, T, 0, s>>>(b);
     return cudaGetLastError();
 }
 
