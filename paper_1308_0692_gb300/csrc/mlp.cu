@@ -1,10 +1,11 @@
 // Learned warm start: a coordinate MLP 4 -> 256 -> 256 -> 256 -> 6 (exact-erf GELU) that
 // maps (x, y, log Kn, u_w) to the six normalised moments of the steady state, trained
-// and evaluated with this file's kernels: BF16 GEMMs on the fifth-generation tensor cores
-// with FP32 accumulation in tensor memory (umma_gemm.cu: TMA tensor copies, tcgen05.mma,
-// tcgen05.ld; split-K with a fixed-order sum for the weight gradients, whose K is the
-// batch), elementwise GELU / GELU' / loss kernels, bias-gradient reductions and Adam on
-// FP32 master weights.  The warm-start kernel then builds the initial distribution
+// and evaluated on the fifth-generation tensor cores in BF16 with FP32 accumulation.  A
+// training step is three launches: the row-local chain (forward pass, loss, input gradients;
+// mlp_chain.cu), the weight gradients, and their reduction with Adam on FP32 master weights
+// (mlp_grad.cu); a forward pass is the chain alone.  As one launch per product, activation,
+// transposition, column sum and array update a training step of 8192 rows took 390 us.  The
+// warm-start kernel then builds the initial distribution
 // from the predicted moments by the second-order Hermite expansion
 //   h_a = w_a [rho' + xi_a . j' + 1/2 sum_ij (P'_ij - rho' delta_ij)(xi_i xi_j - delta_ij)].
 // The paper has no learned component; this follows the warm-start configuration of
@@ -20,152 +21,22 @@
 
 #include "../../include/lbm.h"
 #include "lbm_internal.h"
+#include "mlp_internal.h"
+#include "umma.cuh"
 
 lbm_status lbm_norms_fail(lbm_status s, const char *msg);
 
-// tensor-core GEMM (umma_gemm.cu)
-cudaError_t umma_gemm_nt(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb, float *C, int ldc,
-                         const float *bias, int M, int N, int K, int splits, float *partials, int *status,
-                         cudaStream_t s);
+using namespace mlpk;
 
 namespace {
 
-constexpr int NL = 4;                          // layers
-constexpr int WIDTH[NL + 1] = {4, 256, 256, 256, 6};
-constexpr int PADW[NL + 1] = {8, 256, 256, 256, 8};   // row lengths padded to 16 bytes
-constexpr int SPLITK_MAX = 32;                        // K-splits of a weight-gradient GEMM
-
-// ------------------------------------------------------------------ elementwise kernels
-__device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad_f(float z)
+// both BF16 copies of a layer's weights W [N][K]: q [N][ldq] and its transpose qt [K][ldt]
+__global__ void refresh_kernel(const float *W, int n, int k, __nv_bfloat16 *q, int ldq, __nv_bfloat16 *qt, int ldt)
 {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
-}
-
-// dst[r][c] (bf16, ld = ldd) = src[r][c] (fp32, ld = lds) for c < cols, 0 for cols <= c < ldd
-__global__ void to_bf16_kernel(const float *src, int lds, __nv_bfloat16 *dst, int ldd, int rows, int cols)
-{
-    const long n = (long)rows * ldd;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const int r = (int)(i / ldd), c = (int)(i - (long)r * ldd);
-        dst[i] = __float2bfloat16_rn(c < cols ? src[(long)r * lds + c] : 0.f);
-    }
-}
-
-// a = bf16(GELU(z)) for a [rows][cols] block (z ld = cols, a ld = lda, padding zeroed)
-__global__ void gelu_fwd_kernel(const float *z, __nv_bfloat16 *a, int lda, int rows, int cols)
-{
-    const long n = (long)rows * lda;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const int r = (int)(i / lda), c = (int)(i - (long)r * lda);
-        a[i] = __float2bfloat16_rn(c < cols ? gelu_f(z[(long)r * cols + c]) : 0.f);
-    }
-}
-
-// g = bf16(da * GELU'(z))
-__global__ void gelu_bwd_kernel(const float *da, const float *z, __nv_bfloat16 *g, float *g32, long n)
-{
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const float v = da[i] * gelu_grad_f(z[i]);
-        g32[i] = v;
-        g[i] = __float2bfloat16_rn(v);
-    }
-}
-
-// output-layer gradient g = 2 (y - t) / (M * nout) (fp32 and bf16 padded to ldg), and
-// per-block partial sums of (y - t)^2
-__global__ void loss_grad_kernel(const float *y, const float *t, int M, int nout, float *g32,
-                                 __nv_bfloat16 *g16, int ldg, double *partials)
-{
-    __shared__ double s[8];
-    double acc = 0.0;
-    const float scale = 2.0f / ((float)M * (float)nout);
-    const long n = (long)M * ldg;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const int r = (int)(i / ldg), c = (int)(i - (long)r * ldg);
-        float gv = 0.f;
-        if (c < nout) {
-            const float d = y[(long)r * nout + c] - t[(long)r * nout + c];
-            acc += (double)d * d;
-            gv = scale * d;
-            g32[(long)r * nout + c] = gv;
-        }
-        g16[i] = __float2bfloat16_rn(gv);
-    }
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < 8; ++w) tot += s[w];
-        partials[blockIdx.x] = tot;
-    }
-}
-
-// dst[c][r] = src[r][c] (bf16), src [rows][ld_src] -> dst [cols][ld_dst] (padding zeroed)
-__global__ void transpose_bf16_kernel(const __nv_bfloat16 *src, int lds, __nv_bfloat16 *dst, int ldd, int rows,
-                                      int cols, int dst_rows)
-{
-    __shared__ __nv_bfloat16 tile[32][33];
-    const int bx = blockIdx.x * 32, by = blockIdx.y * 32;   // bx over src cols, by over src rows
-    for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-        const int r = by + j, c = bx + threadIdx.x;
-        tile[j][threadIdx.x] = (r < rows && c < cols) ? src[(long)r * lds + c] : __float2bfloat16_rn(0.f);
-    }
-    __syncthreads();
-    for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-        const int c = bx + j, r = by + threadIdx.x;   // dst row c, dst col r
-        if (c < dst_rows && r < ldd) dst[(long)c * ldd + r] = tile[threadIdx.x][j];
-    }
-}
-
-// db[c] = sum_r g[r][c] (fp32, fixed order): block (x, y) sums rows [y*chunk, (y+1)*chunk)
-// of columns [32x, 32x+32), lane = column (coalesced reads), warps over rows; the second
-// kernel adds the row chunks in order.  At most CS_CHUNKS chunks (of at least 256 rows).
-constexpr int CS_CHUNKS = 2048;
-__global__ void __launch_bounds__(256) colsum_part_kernel(const float *g, int rows, int cols, int chunk, float *part)
-{
-    __shared__ float s[8][33];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int c = blockIdx.x * 32 + lane;
-    const int r0 = blockIdx.y * chunk, r1 = min(rows, r0 + chunk);
-    float acc = 0.f;
-    if (c < cols)
-        for (int r = r0 + w; r < r1; r += 8) acc += g[(long)r * cols + c];
-    s[w][lane] = acc;
-    __syncthreads();
-    if (w == 0 && c < cols) {
-        float t = 0.f;
-        for (int q = 0; q < 8; ++q) t += s[q][lane];
-        part[(long)blockIdx.y * cols + c] = t;
-    }
-}
-
-__global__ void colsum_final_kernel(const float *part, int chunks, int cols, float *db)
-{
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-    float t = 0.f;
-    for (int k = 0; k < chunks; ++k) t += part[(long)k * cols + c];
-    db[c] = t;
-}
-
-// Adam on FP32 master weights; refreshes the bf16 copy (ld = ldq, row length k)
-__global__ void adam_kernel(float *p, const float *gr, float *m, float *v, long n, int k, __nv_bfloat16 *q,
-                            int ldq, float lr, float b1, float b2, float eps, float c1, float c2)
-{
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const float g = gr[i];
-        const float mi = b1 * m[i] + (1.f - b1) * g;
-        const float vi = b2 * v[i] + (1.f - b2) * g * g;
-        m[i] = mi;
-        v[i] = vi;
-        const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-        p[i] = pi;
-        if (q) {
-            const int r = (int)(i / k), c = (int)(i - (long)r * k);
-            q[(long)r * ldq + c] = __float2bfloat16_rn(pi);
-        }
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * k; i += gridDim.x * blockDim.x) {
+        const __nv_bfloat16 v = __float2bfloat16_rn(W[i]);
+        q[(i / k) * ldq + i % k] = v;
+        qt[(i % k) * ldt + i / k] = v;
     }
 }
 
@@ -220,25 +91,22 @@ lbm_status mfail(lbm_status s, const std::string &m) { return lbm_norms_fail(s, 
 
 struct lbm_mlp {
     int max_batch;
+    long ld;                  // row pitch of the transposed operands: max_batch in whole row tiles
     cudaStream_t stream;
     void *base;
-    // parameters (FP32 master, bf16 copies, Adam moments) and gradients, per layer
-    float *W[NL], *b[NL], *gW[NL], *gb[NL], *mW[NL], *vW[NL], *mb[NL], *vb[NL];
-    __nv_bfloat16 *Wq[NL];    // [N][PADW[l]]
-    __nv_bfloat16 *WqT[NL];   // [K][PADW[l+1]] (transposed copy for the input gradient)
-    // activations for max_batch rows
-    float *x32;               // staging of inputs
-    __nv_bfloat16 *a[NL];     // layer inputs, bf16 [M][PADW[l]]
-    float *z[NL];             // pre-activations [M][WIDTH[l+1]]
-    float *g32;               // gradient w.r.t. z of the current layer [M][256]
-    __nv_bfloat16 *g16;       // same, bf16 [M][256 or 8 padded]
-    float *da;                // gradient w.r.t. a [M][256]
-    __nv_bfloat16 *gT;        // transposed g [256][M]
-    __nv_bfloat16 *aT;        // transposed a [256][M]
+    // flat parameters (W_0, b_0, W_1, ...), Adam moments and gradient; BF16 copies per layer
+    float *p, *m, *v, *grad;
+    __nv_bfloat16 *wq[NL];    // [N][PADW[l]]
+    __nv_bfloat16 *wqT[NL];   // [K][PADW[l+1]]
+    float *x32;               // staging of a forward pass in place
+    __nv_bfloat16 *aT[NL], *gT[NL];
+    float *gp, *colpart, *part;
     double *loss_part;
     double *host_loss;
-    float *splitk;            // split-K partial tiles of the weight-gradient GEMMs
-    int *status;              // set by a tensor-core GEMM whose bounded wait gave up
+    int *status;              // set by a kernel whose bounded wait gave up
+    ChainMaps chain;
+    GradMaps grads;           // of grad_tiles row tiles
+    int grad_tiles;
     long step;
 };
 
@@ -246,132 +114,103 @@ namespace {
 
 size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 
+constexpr long nparams()
+{
+    long n = 0;
+    for (int l = 0; l < NL; ++l) n += (long)WIDTH[l + 1] * WIDTH[l] + WIDTH[l + 1];
+    return n;
+}
+
+// offset of layer l's weights in the flat arrays; its biases follow them
+long weights_at(int l)
+{
+    long o = 0;
+    for (int q = 0; q < l; ++q) o += (long)WIDTH[q + 1] * WIDTH[q] + WIDTH[q + 1];
+    return o;
+}
+long biases_at(int l) { return weights_at(l) + (long)WIDTH[l + 1] * WIDTH[l]; }
+
+int row_tiles(int rows) { return (rows + ROWS - 1) / ROWS; }
+
 // layout of all device arrays of one MLP; returns total bytes, fills pointers if base != nullptr
 size_t mlp_layout(lbm_mlp *p, char *base, int M)
 {
     size_t off = 0;
+    const long tiles = row_tiles(M), ld = tiles * ROWS;
     auto take = [&](size_t bytes) -> char * {
         char *r = base ? base + off : nullptr;
         off = al(off + bytes);
         return r;
     };
+    lbm_mlp dummy;
+    lbm_mlp &q = p ? *p : dummy;
+    q.ld = ld;
+    for (float **f : {&q.p, &q.m, &q.v, &q.grad}) *f = (float *)take(4 * nparams());
     for (int l = 0; l < NL; ++l) {
-        const size_t nw = (size_t)WIDTH[l + 1] * WIDTH[l], nb = WIDTH[l + 1];
-        float *W = (float *)take(4 * nw), *b = (float *)take(4 * nb), *gW = (float *)take(4 * nw), *gb = (float *)take(4 * nb);
-        float *mW = (float *)take(4 * nw), *vW = (float *)take(4 * nw), *mb = (float *)take(4 * nb), *vb = (float *)take(4 * nb);
-        __nv_bfloat16 *Wq = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l + 1] * PADW[l]);
-        __nv_bfloat16 *WqT = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l] * PADW[l + 1]);
-        __nv_bfloat16 *a = (__nv_bfloat16 *)take(2 * (size_t)M * PADW[l]);
-        float *z = (float *)take(4 * (size_t)M * WIDTH[l + 1]);
-        if (p) {
-            p->W[l] = W; p->b[l] = b; p->gW[l] = gW; p->gb[l] = gb;
-            p->mW[l] = mW; p->vW[l] = vW; p->mb[l] = mb; p->vb[l] = vb;
-            p->Wq[l] = Wq; p->WqT[l] = WqT; p->a[l] = a; p->z[l] = z;
-        }
+        q.wq[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l + 1] * PADW[l]);
+        q.wqT[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l] * PADW[l + 1]);
+        q.aT[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l] * ld);
+        q.gT[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l + 1] * ld);
     }
-    float *x32 = (float *)take(4 * (size_t)M * 4);
-    float *g32 = (float *)take(4 * (size_t)M * 256);
-    __nv_bfloat16 *g16 = (__nv_bfloat16 *)take(2 * (size_t)M * 256);
-    float *da = (float *)take(4 * (size_t)M * 256);
-    __nv_bfloat16 *gT = (__nv_bfloat16 *)take(2 * (size_t)256 * (M + 8));
-    __nv_bfloat16 *aT = (__nv_bfloat16 *)take(2 * (size_t)256 * (M + 8));
-    double *lp = (double *)take(8 * 1216);
-    // split-K partial tiles (<= SPLITK_MAX x 256 x 256), also the column sums' chunk partials
-    // (<= CS_CHUNKS x 256)
-    float *sk = (float *)take(4 * (size_t)SPLITK_MAX * 256 * 256);
-    static_assert(CS_CHUNKS * 256 <= SPLITK_MAX * 256 * 256, "workspace too small for the column sums");
-    int *stw = (int *)take(16);
-    if (p) {
-        p->x32 = x32; p->g32 = g32; p->g16 = g16; p->da = da; p->gT = gT; p->aT = aT; p->loss_part = lp;
-        p->splitk = sk; p->status = stw;
-    }
+    q.x32 = (float *)take(16 * (size_t)M);
+    q.gp = (float *)take(4 * (size_t)3 * 256 * ld);
+    q.colpart = (float *)take(4 * (size_t)COLS * tiles);
+    q.part = (float *)take(4 * (size_t)WTILES * SPLITS * 128 * 128);
+    q.loss_part = (double *)take(8 * (size_t)tiles);
+    q.status = (int *)take(16);
     return off;
 }
 
 int blocks_for(long n) { long b = (n + 255) / 256; return (int)(b < 1 ? 1 : (b > 1216 ? 1216 : b)); }
 
-// C[M][N] = A[M][K] B[N][K]^T (+ bias) on the tensor cores; K-splits for long K (the batch)
-cudaError_t gemm(lbm_mlp *p, const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb, float *C, int ldc,
-                 const float *bias, int M, int N, int K)
-{
-    const int ktiles = (K + 63) / 64;
-    int splits = ktiles / 4;
-    if (splits > SPLITK_MAX) splits = SPLITK_MAX;
-    if (splits < 2 || (long)M * N > 256L * 256) splits = 1;
-    return umma_gemm_nt(A, lda, B, ldb, C, ldc, bias, M, N, K, splits, p->splitk, p->status, p->stream);
-}
-
 cudaError_t refresh_bf16(lbm_mlp *p, int l)
 {
-    cudaError_t e = cudaSuccess;
-    to_bf16_kernel<<<blocks_for((long)WIDTH[l + 1] * PADW[l]), 256, 0, p->stream>>>(p->W[l], WIDTH[l], p->Wq[l], PADW[l],
-                                                                                   WIDTH[l + 1], WIDTH[l]);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    dim3 tg((PADW[l] + 31) / 32, (WIDTH[l + 1] + 31) / 32);
-    // WqT [K][PADW[l+1]] = Wq^T; rows of WqT = K = WIDTH[l]
-    transpose_bf16_kernel<<<tg, dim3(32, 8), 0, p->stream>>>(p->Wq[l], PADW[l], p->WqT[l], PADW[l + 1], WIDTH[l + 1],
-                                                            PADW[l], WIDTH[l]);
+    const int n = WIDTH[l + 1], k = WIDTH[l];
+    refresh_kernel<<<blocks_for((long)n * k), 256, 0, p->stream>>>(p->p + weights_at(l), n, k, p->wq[l], PADW[l], p->wqT[l],
+                                                                   PADW[l + 1]);
     return cudaGetLastError();
 }
 
-// forward pass on M rows already staged in p->x32; leaves y in p->z[NL-1] [M][6]
-cudaError_t forward(lbm_mlp *p, int M)
+bool make_chain_maps(lbm_mlp *p)
 {
-    cudaStream_t s = p->stream;
-    to_bf16_kernel<<<blocks_for((long)M * PADW[0]), 256, 0, s>>>(p->x32, 4, p->a[0], PADW[0], M, 4);
-    cudaError_t e = cudaGetLastError();
-    for (int l = 0; l < NL && e == cudaSuccess; ++l) {
-        e = gemm(p, p->a[l], PADW[l], p->Wq[l], PADW[l], p->z[l], WIDTH[l + 1], p->b[l], M, WIDTH[l + 1], PADW[l]);
-        if (e == cudaSuccess && l + 1 < NL) {
-            gelu_fwd_kernel<<<blocks_for((long)M * PADW[l + 1]), 256, 0, s>>>(p->z[l], p->a[l + 1], PADW[l + 1], M,
-                                                                            WIDTH[l + 1]);
-            e = cudaGetLastError();
-        }
-    }
-    return e;
+    bool ok = true;
+    for (int l = 0; l < NL; ++l)
+        ok = ok && umma::make_map(&p->chain.w[l], p->wq[l], WIDTH[l + 1], PADW[l], PADW[l], l == 3 ? 16 : 128);
+    for (int l = NL - 1; l > 0; --l)
+        ok = ok && umma::make_map(&p->chain.w[7 - l], p->wqT[l], WIDTH[l], PADW[l + 1], PADW[l + 1], 128);
+    return ok;
 }
 
-// backward pass after forward(); targets t [M][6] on device; fills gW, gb and loss partials
-cudaError_t backward(lbm_mlp *p, const float *t, int M, int *nparts)
+// the weight gradients sum over whole row tiles: their maps end at the batch's last one
+bool make_grad_maps(lbm_mlp *p, int tiles)
 {
-    cudaStream_t s = p->stream;
-    const int nb = blocks_for((long)M * PADW[NL]);
-    loss_grad_kernel<<<nb, 256, 0, s>>>(p->z[NL - 1], t, M, WIDTH[NL], p->g32, p->g16, PADW[NL], p->loss_part);
-    *nparts = nb;
-    cudaError_t e = cudaGetLastError();
-    int ldg = PADW[NL];            // row length of the bf16 gradient g16
-    int ng = WIDTH[NL];            // columns of the fp32 gradient g32
-    for (int l = NL - 1; l >= 0 && e == cudaSuccess; --l) {
-        // gW[l] [N][K] = g^T a_l : A = g^T [N][M], B = a_l^T [K][M]
-        const int Mp = ((M + 7) / 8) * 8;
-        dim3 tg1((ldg + 31) / 32, (M + 31) / 32);
-        transpose_bf16_kernel<<<tg1, dim3(32, 8), 0, s>>>(p->g16, ldg, p->gT, Mp, M, ldg, WIDTH[l + 1]);
-        dim3 tg2((PADW[l] + 31) / 32, (M + 31) / 32);
-        transpose_bf16_kernel<<<tg2, dim3(32, 8), 0, s>>>(p->a[l], PADW[l], p->aT, Mp, M, PADW[l], WIDTH[l]);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = gemm(p, p->gT, Mp, p->aT, Mp, p->gW[l], WIDTH[l], nullptr, WIDTH[l + 1], WIDTH[l], Mp);
-        if (e == cudaSuccess) {
-            // the split-K workspace is free again once the weight-gradient GEMM is done
-            int chunk = (M + CS_CHUNKS - 1) / CS_CHUNKS;
-            if (chunk < 256) chunk = 256;
-            const int chunks = (M + chunk - 1) / chunk;       // <= CS_CHUNKS: fits the workspace
-            colsum_part_kernel<<<dim3((ng + 31) / 32, chunks), 256, 0, s>>>(p->g32, M, ng, chunk, p->splitk);
-            colsum_final_kernel<<<(ng + 255) / 256, 256, 0, s>>>(p->splitk, chunks, ng, p->gb[l]);
-            e = cudaGetLastError();
-        }
-        if (l == 0 || e != cudaSuccess) break;
-        // da [M][K] = g W : A = g [M][N] (bf16 ld ldg), B = W^T [K][N] (WqT, ld PADW[l+1])
-        e = gemm(p, p->g16, ldg, p->WqT[l], PADW[l + 1], p->da, WIDTH[l], nullptr, M, WIDTH[l], ldg);
-        if (e == cudaSuccess) {
-            const long n = (long)M * WIDTH[l];
-            gelu_bwd_kernel<<<blocks_for(n), 256, 0, s>>>(p->da, p->z[l - 1], p->g16, p->g32, n);
-            e = cudaGetLastError();
-        }
-        ldg = WIDTH[l];
-        ng = WIDTH[l];
+    if (p->grad_tiles == tiles) return true;
+    p->grad_tiles = 0;
+    bool ok = true;
+    for (int l = 0; l < NL; ++l)
+        ok = ok && umma::make_map(&p->grads.g[l], p->gT[l], WIDTH[l + 1], (long)tiles * ROWS, p->ld, 128) &&
+             umma::make_map(&p->grads.a[l], p->aT[l], WIDTH[l], (long)tiles * ROWS, p->ld, l == 0 ? 16 : 128);
+    if (ok) p->grad_tiles = tiles;
+    return ok;
+}
+
+ChainArgs chain_args(lbm_mlp *p, const float *x, int M)
+{
+    ChainArgs a;
+    std::memset(&a, 0, sizeof a);
+    a.x = x;
+    for (int l = 0; l < NL; ++l) {
+        a.b[l] = p->p + biases_at(l);
+        a.aT[l] = p->aT[l];
+        a.gT[l] = p->gT[l];
     }
-    return e;
+    a.gp = p->gp;
+    a.colpart = p->colpart;
+    a.loss = p->loss_part;
+    a.ld = p->ld;
+    a.M = M;
+    a.status = p->status;
+    return a;
 }
 
 // splitmix64-based uniform numbers for the default initialisation
@@ -391,9 +230,7 @@ extern "C" {
 lbm_status lbm_mlp_param_count(long *count)
 {
     if (!count) return mfail(LBM_EINVAL, "count is NULL");
-    long n = 0;
-    for (int l = 0; l < NL; ++l) n += (long)WIDTH[l + 1] * WIDTH[l] + WIDTH[l + 1];
-    *count = n;
+    *count = nparams();
     return LBM_OK;
 }
 
@@ -414,7 +251,10 @@ lbm_status lbm_mlp_create(int max_batch, unsigned long long seed, void *stream, 
     }
     mlp_layout(p, (char *)p->base, max_batch);
     e = cudaMemsetAsync(p->base, 0, bytes, p->stream);
-    if (e == cudaSuccess) e = cudaMallocHost(&p->host_loss, sizeof(double) * 1216);
+    if (e == cudaSuccess) e = cudaMallocHost(&p->host_loss, sizeof(double) * row_tiles(max_batch));
+    if (e == cudaSuccess) e = prepare_chain();
+    if (e == cudaSuccess) e = prepare_grads();
+    if (e == cudaSuccess && !make_chain_maps(p)) e = cudaErrorInvalidValue;
     if (e != cudaSuccess) {
         lbm_mlp_destroy(p);
         return mfail(LBM_ECUDA, cudaGetErrorString(e));
@@ -449,20 +289,10 @@ void lbm_mlp_destroy(lbm_mlp *p)
 lbm_status lbm_mlp_set_params(lbm_mlp *p, const float *flat)
 {
     if (!p || !flat) return mfail(LBM_EINVAL, "NULL argument");
-    long o = 0;
-    cudaError_t e = cudaSuccess;
-    for (int l = 0; l < NL && e == cudaSuccess; ++l) {
-        const long nw = (long)WIDTH[l + 1] * WIDTH[l];
-        e = cudaMemcpyAsync(p->W[l], flat + o, 4 * nw, cudaMemcpyHostToDevice, p->stream);
-        o += nw;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(p->b[l], flat + o, 4 * WIDTH[l + 1], cudaMemcpyHostToDevice, p->stream);
-        o += WIDTH[l + 1];
-        if (e == cudaSuccess) e = cudaMemsetAsync(p->mW[l], 0, 4 * nw, p->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(p->vW[l], 0, 4 * nw, p->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(p->mb[l], 0, 4 * WIDTH[l + 1], p->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(p->vb[l], 0, 4 * WIDTH[l + 1], p->stream);
-        if (e == cudaSuccess) e = refresh_bf16(p, l);
-    }
+    cudaError_t e = cudaMemcpyAsync(p->p, flat, 4 * nparams(), cudaMemcpyHostToDevice, p->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->m, 0, 4 * nparams(), p->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->v, 0, 4 * nparams(), p->stream);
+    for (int l = 0; l < NL && e == cudaSuccess; ++l) e = refresh_bf16(p, l);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
     p->step = 0;
     return e == cudaSuccess ? LBM_OK : mfail(LBM_ECUDA, cudaGetErrorString(e));
@@ -471,15 +301,7 @@ lbm_status lbm_mlp_set_params(lbm_mlp *p, const float *flat)
 lbm_status lbm_mlp_get_params(lbm_mlp *p, float *flat)
 {
     if (!p || !flat) return mfail(LBM_EINVAL, "NULL argument");
-    long o = 0;
-    cudaError_t e = cudaSuccess;
-    for (int l = 0; l < NL && e == cudaSuccess; ++l) {
-        const long nw = (long)WIDTH[l + 1] * WIDTH[l];
-        e = cudaMemcpyAsync(flat + o, p->W[l], 4 * nw, cudaMemcpyDeviceToHost, p->stream);
-        o += nw;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(flat + o, p->b[l], 4 * WIDTH[l + 1], cudaMemcpyDeviceToHost, p->stream);
-        o += WIDTH[l + 1];
-    }
+    cudaError_t e = cudaMemcpyAsync(flat, p->p, 4 * nparams(), cudaMemcpyDeviceToHost, p->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
     return e == cudaSuccess ? LBM_OK : mfail(LBM_ECUDA, cudaGetErrorString(e));
 }
@@ -487,47 +309,72 @@ lbm_status lbm_mlp_get_params(lbm_mlp *p, float *flat)
 lbm_status lbm_mlp_forward(lbm_mlp *p, const float *x_dev, int M, float *y_dev)
 {
     if (!p || !x_dev || !y_dev || M < 1 || M > p->max_batch) return mfail(LBM_EINVAL, "invalid forward arguments");
-    cudaError_t e = cudaMemcpyAsync(p->x32, x_dev, 16L * M, cudaMemcpyDeviceToDevice, p->stream);
-    if (e == cudaSuccess) e = forward(p, M);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(y_dev, p->z[NL - 1], 24L * M, cudaMemcpyDeviceToDevice, p->stream);
+    // row tiles write y while others still read x: overlapping buffers go through a copy of x
+    const uintptr_t x0 = (uintptr_t)x_dev, y0 = (uintptr_t)y_dev;
+    cudaError_t e = cudaSuccess;
+    if (x0 < y0 + 24L * M && y0 < x0 + 16L * M) {
+        e = cudaMemcpyAsync(p->x32, x_dev, 16L * M, cudaMemcpyDeviceToDevice, p->stream);
+        x_dev = p->x32;
+    }
+    ChainArgs a = chain_args(p, x_dev, M);
+    a.y = y_dev;
+    if (e == cudaSuccess) e = launch_chain(false, p->chain, a, p->stream);
     return e == cudaSuccess ? LBM_OK : mfail(LBM_ECUDA, cudaGetErrorString(e));
 }
 
-static lbm_status grads_and_loss(lbm_mlp *p, const float *x_dev, const float *t_dev, int M, double *loss)
+// Chain, weight gradients and their reduction: the gradient into p->grad (lr = 0) or one Adam
+// step; the loss (may be NULL) of the parameters before it.
+static lbm_status train(lbm_mlp *p, const float *x_dev, const float *t_dev, int M, float lr, double *loss)
 {
-    cudaError_t e = cudaMemcpyAsync(p->x32, x_dev, 16L * M, cudaMemcpyDeviceToDevice, p->stream);
-    if (e == cudaSuccess) e = forward(p, M);
-    int np = 0;
-    if (e == cudaSuccess) e = backward(p, t_dev, M, &np);
+    const int tiles = row_tiles(M), ktiles = tiles * (ROWS / umma::UK), splits = ktiles < SPLITS ? ktiles : SPLITS;
+    if (!make_grad_maps(p, tiles)) return mfail(LBM_ECUDA, "encoding a tensor map failed");
+    ChainArgs c = chain_args(p, x_dev, M);
+    c.t = t_dev;
+    cudaError_t e = launch_chain(true, p->chain, c, p->stream);
+    if (e == cudaSuccess) e = launch_grads(p->grads, ktiles, splits, p->part, p->status, p->stream);
     if (e != cudaSuccess) return mfail(LBM_ECUDA, cudaGetErrorString(e));
     if (loss) {
         int stw = 0;
-        e = cudaMemcpyAsync(p->host_loss, p->loss_part, 8L * np, cudaMemcpyDeviceToHost, p->stream);
+        e = cudaMemcpyAsync(p->host_loss, p->loss_part, 8L * tiles, cudaMemcpyDeviceToHost, p->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&stw, p->status, sizeof(int), cudaMemcpyDeviceToHost, p->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
         if (e != cudaSuccess) return mfail(LBM_ECUDA, cudaGetErrorString(e));
-        if (stw != 0) return mfail(LBM_ETIMEOUT, "a bounded wait of the tensor-core GEMM gave up");
+        if (stw != 0) return mfail(LBM_ETIMEOUT, "a bounded wait of a tensor-core kernel gave up");
         double s = 0.0;
-        for (int i = 0; i < np; ++i) s += p->host_loss[i];
+        for (int i = 0; i < tiles; ++i) s += p->host_loss[i];
         *loss = s / ((double)M * WIDTH[NL]);
     }
-    return LBM_OK;
+    AdamArgs a;
+    std::memset(&a, 0, sizeof a);
+    a.part = p->part;
+    a.colpart = p->colpart;
+    a.splits = splits;
+    a.tiles = tiles;
+    if (lr > 0) {
+        p->step += 1;
+        a.p = p->p;
+        a.m = p->m;
+        a.v = p->v;
+        for (int l = 0; l < NL; ++l) {
+            a.wq[l] = p->wq[l];
+            a.wqT[l] = p->wqT[l];
+        }
+        a.lr = lr;
+        a.c1 = 1.f - std::pow(0.9f, (float)p->step);
+        a.c2 = 1.f - std::pow(0.999f, (float)p->step);
+    } else {
+        a.grad = p->grad;
+    }
+    e = launch_reduce_adam(a, p->stream);
+    return e == cudaSuccess ? LBM_OK : mfail(LBM_ECUDA, cudaGetErrorString(e));
 }
 
 lbm_status lbm_mlp_loss_grad(lbm_mlp *p, const float *x_dev, const float *t_dev, int M, double *loss, float *grad_flat)
 {
     if (!p || !x_dev || !t_dev || M < 1 || M > p->max_batch) return mfail(LBM_EINVAL, "invalid arguments");
-    lbm_status st = grads_and_loss(p, x_dev, t_dev, M, loss);
+    lbm_status st = train(p, x_dev, t_dev, M, 0.f, loss);
     if (st != LBM_OK || !grad_flat) return st;
-    long o = 0;
-    cudaError_t e = cudaSuccess;
-    for (int l = 0; l < NL && e == cudaSuccess; ++l) {
-        const long nw = (long)WIDTH[l + 1] * WIDTH[l];
-        e = cudaMemcpyAsync(grad_flat + o, p->gW[l], 4 * nw, cudaMemcpyDeviceToHost, p->stream);
-        o += nw;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(grad_flat + o, p->gb[l], 4 * WIDTH[l + 1], cudaMemcpyDeviceToHost, p->stream);
-        o += WIDTH[l + 1];
-    }
+    cudaError_t e = cudaMemcpyAsync(grad_flat, p->grad, 4 * nparams(), cudaMemcpyDeviceToHost, p->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
     return e == cudaSuccess ? LBM_OK : mfail(LBM_ECUDA, cudaGetErrorString(e));
 }
@@ -535,22 +382,7 @@ lbm_status lbm_mlp_loss_grad(lbm_mlp *p, const float *x_dev, const float *t_dev,
 lbm_status lbm_mlp_train_step(lbm_mlp *p, const float *x_dev, const float *t_dev, int M, float lr, double *loss)
 {
     if (!p || !x_dev || !t_dev || M < 1 || M > p->max_batch || !(lr > 0)) return mfail(LBM_EINVAL, "invalid arguments");
-    lbm_status st = grads_and_loss(p, x_dev, t_dev, M, loss);
-    if (st != LBM_OK) return st;
-    p->step += 1;
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = 1.f - std::pow(b1, (float)p->step), c2 = 1.f - std::pow(b2, (float)p->step);
-    cudaError_t e = cudaSuccess;
-    for (int l = 0; l < NL && e == cudaSuccess; ++l) {
-        const long nw = (long)WIDTH[l + 1] * WIDTH[l];
-        adam_kernel<<<blocks_for(nw), 256, 0, p->stream>>>(p->W[l], p->gW[l], p->mW[l], p->vW[l], nw, WIDTH[l],
-                                                           nullptr, 0, lr, b1, b2, eps, c1, c2);
-        adam_kernel<<<1, 256, 0, p->stream>>>(p->b[l], p->gb[l], p->mb[l], p->vb[l], WIDTH[l + 1], WIDTH[l + 1],
-                                              nullptr, 0, lr, b1, b2, eps, c1, c2);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = refresh_bf16(p, l);
-    }
-    return e == cudaSuccess ? LBM_OK : mfail(LBM_ECUDA, cudaGetErrorString(e));
+    return train(p, x_dev, t_dev, M, lr, loss);
 }
 
 lbm_status lbm_mlp_features(lbm_mlp *p, int nx, int ny, double kn, double u_w, float *x_dev)
