@@ -91,7 +91,6 @@ lbm_status mfail(lbm_status s, const std::string &m) { return lbm_norms_fail(s, 
 
 struct lbm_mlp {
     int max_batch;
-    long ld;                  // row pitch of the transposed operands: max_batch in whole row tiles
     cudaStream_t stream;
     void *base;
     // flat parameters (W_0, b_0, W_1, ...), Adam moments and gradient; BF16 copies per layer
@@ -136,7 +135,7 @@ int row_tiles(int rows) { return (rows + ROWS - 1) / ROWS; }
 size_t mlp_layout(lbm_mlp *p, char *base, int M)
 {
     size_t off = 0;
-    const long tiles = row_tiles(M), ld = tiles * ROWS;
+    const long tiles = row_tiles(M), rows = tiles * ROWS;
     auto take = [&](size_t bytes) -> char * {
         char *r = base ? base + off : nullptr;
         off = al(off + bytes);
@@ -144,16 +143,15 @@ size_t mlp_layout(lbm_mlp *p, char *base, int M)
     };
     lbm_mlp dummy;
     lbm_mlp &q = p ? *p : dummy;
-    q.ld = ld;
     for (float **f : {&q.p, &q.m, &q.v, &q.grad}) *f = (float *)take(4 * nparams());
     for (int l = 0; l < NL; ++l) {
         q.wq[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l + 1] * PADW[l]);
         q.wqT[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l] * PADW[l + 1]);
-        q.aT[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l] * ld);
-        q.gT[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l + 1] * ld);
+        q.aT[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l] * rows);
+        q.gT[l] = (__nv_bfloat16 *)take(2 * (size_t)WIDTH[l + 1] * rows);
     }
     q.x32 = (float *)take(16 * (size_t)M);
-    q.gp = (float *)take(4 * (size_t)3 * 256 * ld);
+    q.gp = (float *)take(4 * (size_t)3 * 256 * rows);
     q.colpart = (float *)take(4 * (size_t)COLS * tiles);
     q.part = (float *)take(4 * (size_t)WTILES * SPLITS * 128 * 128);
     q.loss_part = (double *)take(8 * (size_t)tiles);
@@ -188,8 +186,8 @@ bool make_grad_maps(lbm_mlp *p, int tiles)
     p->grad_tiles = 0;
     bool ok = true;
     for (int l = 0; l < NL; ++l)
-        ok = ok && umma::make_map(&p->grads.g[l], p->gT[l], WIDTH[l + 1], (long)tiles * ROWS, p->ld, 128) &&
-             umma::make_map(&p->grads.a[l], p->aT[l], WIDTH[l], (long)tiles * ROWS, p->ld, l == 0 ? 16 : 128);
+        ok = ok && umma::make_map(&p->grads.g[l], p->gT[l], WIDTH[l + 1], ROWS, ROWS, 128, tiles) &&
+             umma::make_map(&p->grads.a[l], p->aT[l], WIDTH[l], ROWS, ROWS, l == 0 ? 16 : 128, tiles);
     if (ok) p->grad_tiles = tiles;
     return ok;
 }
@@ -207,7 +205,6 @@ ChainArgs chain_args(lbm_mlp *p, const float *x, int M)
     a.gp = p->gp;
     a.colpart = p->colpart;
     a.loss = p->loss_part;
-    a.ld = p->ld;
     a.M = M;
     a.status = p->status;
     return a;

@@ -17,9 +17,12 @@
 // products, each behind a cluster barrier.  Two CTAs per 128 rows put that work on 128 SMs at
 // 8192 rows instead of 64, and sixteen warps per CTA keep each SM quarter's issue slots busy.
 //
-// Training leaves for the weight gradients the transposed operands a_l^T, g_l^T (lane = row, so
-// a warp's store of one column is contiguous: no transposition pass) and per tile the column
+// Training leaves for the weight gradients the transposed operands a_l^T, g_l^T, row tile by row
+// tile ([tile][column][128]: lane = row, so a warp's store of one column is contiguous and needs
+// no transposition pass, and the columns are a fixed distance apart), and per tile the column
 // sums of the FP32 g_l in a fixed order (a butterfly over the lanes, then the four row groups).
+// Those stores, GELU' and the column sums come after the arrival at the cluster barrier, behind
+// the next product: before it, the barrier's release waited for every one of the stores.
 #include <cstring>
 
 #include "mlp_internal.h"
@@ -36,15 +39,9 @@ constexpr int BN = 128;                             // columns a CTA computes of
 constexpr int SUB = ROWS * 128;                     // bytes of one 64-wide K step of an operand
 constexpr int SMEM_A = 4 * SUB, SMEM = 2 * SMEM_A + 4 * SUB + 1024;
 
-// GELU'(z) and GELU(z) from one error function
-__device__ __forceinline__ float gelu(float z, float &grad)
-{
-    const float e = 1.0f + erff(z * 0.70710678118654752f);
-    grad = 0.5f * e + z * expf(-0.5f * z * z) * 0.39894228040143268f;
-    return 0.5f * z * e;
-}
-
-__device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
+// GELU(z) = z e / 2 with e = 1 + erf(z / sqrt 2), and its derivative
+__device__ __forceinline__ float gelu_e(float z) { return 1.0f + erff(z * 0.70710678118654752f); }
+__device__ __forceinline__ float gelu_grad(float z, float e) { return 0.5f * e + z * expf(-0.5f * z * z) * 0.39894228040143268f; }
 
 __device__ __forceinline__ unsigned peer_address(unsigned addr, unsigned rank)
 {
@@ -53,10 +50,8 @@ __device__ __forceinline__ unsigned peer_address(unsigned addr, unsigned rank)
     return r;
 }
 
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 
 __device__ __forceinline__ unsigned pack(float lo, float hi)
 {
@@ -113,12 +108,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
         at[1 ^ (row & 7)] = make_uint4(0u, 0u, 0u, 0u);
         if (TRAIN && rank == 0)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) p.aT[0][c * p.ld + grow] = __float2bfloat16_rn(f[c]);
+            for (int c = 0; c < 4; ++c) p.aT[0][((long)tile * 4 + c) * ROWS + row] = __float2bfloat16_rn(f[c]);
     }
     asm volatile("fence.proxy.async;\n" ::: "memory");
     fence_before_sync();
     __syncthreads();
-    cluster_sync();                                    // the partner's buffers may be written from here on
+    cluster_arrive();
+    cluster_wait();                                    // the partner's buffers may be written from here on
     fence_after_sync();
     const uint32_t tmem = s_tmem;
 
@@ -133,61 +129,63 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     };
     bool ok = true;
     if (tid == 0) fetch(0);
+    __syncwarp();
+    // products of one thread: operand i in abuf, weights i in wbuf
+    auto multiply = [&](int i) {
+        ok = bar_wait(&full, i & 1) && ok;
+        fence_after_sync();
+        asm volatile("fence.proxy.async;\n" ::: "memory");
+        const unsigned char *abuf = smem + (i & 1) * SMEM_A;
+        const uint32_t idesc = instr_desc(rows_of(i));
+        const int nk = ksteps_of(i), ks = nk == 1 ? 1 : UK / 16;       // K = 16 of layer 0's and 3's operands
+        for (int k = 0; k < nk; ++k) {
+            const uint64_t da = smem_desc(abuf + k * SUB), db = smem_desc(wbuf + k * rows_of(i) * 128);
+            for (int q = 0; q < ks; ++q) mma_bf16(tmem, da + 2 * q, db + 2 * q, idesc, (k | q) ? 1u : 0u);
+        }
+        mma_commit(&done);
+    };
+    if (tid == 0) multiply(0);
+    __syncwarp();
 #pragma unroll 1
     for (int i = 0; i < NPROD; ++i) {
         const bool fwd = i < 4;
         const int l = fwd ? i : 6 - i;                 // layer of z (forward) or of g_l (backward)
         const int n0 = rank * BN + cg * 32;            // this warp's first column of a hidden product
-        unsigned char *abuf = smem + (i & 1) * SMEM_A, *anext = smem + ((i + 1) & 1) * SMEM_A;
-        if (tid == 0) {
-            ok = bar_wait(&full, i & 1) && ok;
-            fence_after_sync();
-            asm volatile("fence.proxy.async;\n" ::: "memory");
-            const uint32_t idesc = instr_desc(rows_of(i));
-            const int nk = ksteps_of(i), ks = nk == 1 ? 1 : UK / 16;   // K = 16 of layer 0's and 3's operands
-            for (int k = 0; k < nk; ++k) {
-                const uint64_t da = smem_desc(abuf + k * SUB), db = smem_desc(wbuf + k * rows_of(i) * 128);
-                for (int q = 0; q < ks; ++q) mma_bf16(tmem, da + 2 * q, db + 2 * q, idesc, (k | q) ? 1u : 0u);
-            }
-            mma_commit(&done);
-        }
+        unsigned char *anext = smem + ((i + 1) & 1) * SMEM_A;
+        float *gpt = TRAIN ? p.gp + (((long)tile * 3 + (l < 3 ? l : 0)) * 256 + n0) * ROWS + row : nullptr;
         float gp[TRAIN ? 32 : 1];
         if (TRAIN && !fwd) {                           // GELU' of this thread's values, stored by it before
-            const float *src = p.gp + (long)(l * 256 + n0) * p.ld + grow;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) gp[TRAIN ? j : 0] = src[(long)j * p.ld];
+            for (int j = 0; j < 32; ++j) gp[TRAIN ? j : 0] = gpt[j * ROWS];
         }
         ok = bar_wait(&done, i & 1) && ok;
+        __syncwarp();
         fence_after_sync();
         if (tid == 0 && i + 1 < NPROD) fetch(i + 1);   // the products have read the last weights
         __syncwarp();
         const uint32_t lanes = tmem + ((uint32_t)(rg * 32) << 16);
+        float v[32], z[TRAIN ? 32 : 1];
+        float g[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        double acc = 0.0;
+        // ---- the next product's operand, here and at the partner ----
         if (i != 3) {
-            float v[32];
             tmem_ld32(lanes + (uint32_t)(cg * 32), v);
             if (fwd) {
                 const float *bias = p.b[i];
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
-                    const float z = v[j] + __ldg(bias + n0 + j);
+                    const float zj = v[j] + __ldg(bias + n0 + j), e = gelu_e(zj);
                     if (TRAIN) {
-                        float g;
-                        v[j] = gelu(z, g);
-                        p.gp[(long)(l * 256 + n0 + j) * p.ld + grow] = g;
-                    } else {
-                        v[j] = gelu(z);
+                        z[TRAIN ? j : 0] = zj;
+                        gp[TRAIN ? j : 0] = e;
                     }
+                    v[j] = 0.5f * zj * e;
                 }
             } else {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) v[j] *= gp[TRAIN ? j : 0];
             }
-            if (TRAIN) {
-                __nv_bfloat16 *out = (fwd ? p.aT[fwd ? i + 1 : 0] : p.gT[l]) + (long)n0 * p.ld + grow;
-#pragma unroll
-                for (int j = 0; j < 32; ++j) out[(long)j * p.ld] = __float2bfloat16_rn(v[j]);
-            }
-            if (i + 1 < NPROD) {                       // the next product's operand, here and at the partner
+            if (i + 1 < NPROD) {
                 const unsigned base = su32(anext + (n0 >> 6) * SUB + row * 128);
                 const unsigned far = peer_address(base, (unsigned)(rank ^ 1));
 #pragma unroll
@@ -199,64 +197,91 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
                     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(far + off), "r"(a), "r"(b), "r"(d), "r"(e) : "memory");
                 }
             }
-            if (TRAIN && !fwd) s_col[i & 1][rg][cg * 32 + lane] = column_sum(v, lane);
         } else if (cg == 0) {
-            float z[8];
-            tmem_ld8(lanes, z);
-            float g[6];
-            double acc = 0.0;
+            float y[8];
+            tmem_ld8(lanes, y);
             const float scale = 2.0f / ((float)p.M * 6.0f);
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
-                const float y = z[c] + __ldg(p.b[3] + c);
-                g[c] = 0.f;
+                y[c] += __ldg(p.b[3] + c);
                 if (!TRAIN) {
-                    if (valid && rank == 0) p.y[grow * 6 + c] = y;
-                } else {
-                    if (valid) {
-                        const float d = y - p.t[grow * 6 + c];
-                        acc += (double)d * d;
-                        g[c] = scale * d;
-                    }
-                    if (rank == 0) p.gT[3][c * p.ld + grow] = __float2bfloat16_rn(g[c]);
+                    if (valid && rank == 0) p.y[grow * 6 + c] = y[c];
+                } else if (valid) {
+                    const float d = y[c] - p.t[grow * 6 + c];
+                    acc += (double)d * d;
+                    g[c] = scale * d;
                 }
             }
             if (TRAIN) {
                 uint4 *at = reinterpret_cast<uint4 *>(anext + row * 128);
                 at[0 ^ (row & 7)] = make_uint4(pack(g[0], g[1]), pack(g[2], g[3]), pack(g[4], g[5]), 0u);
                 at[1 ^ (row & 7)] = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    acc += __shfl_xor_sync(0xffffffffu, acc, o);
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) g[c] += __shfl_xor_sync(0xffffffffu, g[c], o);
-                }
-                if (lane == 0) {
-                    s_loss[rg] = acc;
-#pragma unroll
-                    for (int c = 0; c < 6; ++c) s_col[i & 1][rg][c] = g[c];
-                }
             }
         }
         asm volatile("fence.proxy.async;\n" ::: "memory");
         fence_before_sync();
         __syncwarp();
-        cluster_sync();                                // operands complete in both CTAs, accumulator read
-        fence_after_sync();
-        if (TRAIN && (i == 3 ? (rank == 0 && tid < 6) : (!fwd && tid < BN))) {
-            float t = 0.f;
+        cluster_arrive();                              // operands written and the accumulator read
+        if (warp == 0) {
+            cluster_wait();
+            fence_after_sync();
+            if (tid == 0 && i + 1 < NPROD) multiply(i + 1);
+            __syncwarp();
+        }
+        // ---- what the weight gradients need, behind the next product ----
+        if (TRAIN && i != 3) {
+            __nv_bfloat16 *out = (fwd ? p.aT[fwd ? i + 1 : 0] : p.gT[l]) + ((long)tile * 256 + n0) * ROWS + row;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) t += s_col[i & 1][q][tid];
-            p.colpart[(long)tile * COLS + (i == 3 ? 768 : l * 256 + rank * BN) + tid] = t;
-            if (i == 3 && tid == 0) p.loss[tile] = (s_loss[0] + s_loss[1]) + (s_loss[2] + s_loss[3]);
+            for (int j = 0; j < 32; ++j) out[j * ROWS] = __float2bfloat16_rn(v[j]);
+            if (fwd) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) gpt[j * ROWS] = gelu_grad(z[TRAIN ? j : 0], gp[TRAIN ? j : 0]);
+            } else {
+                s_col[i & 1][rg][cg * 32 + lane] = column_sum(v, lane);
+            }
+        } else if (TRAIN && cg == 0) {
+            if (rank == 0)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) p.gT[3][((long)tile * 6 + c) * ROWS + row] = __float2bfloat16_rn(g[c]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                acc += __shfl_xor_sync(0xffffffffu, acc, o);
+#pragma unroll
+                for (int c = 0; c < 6; ++c) g[c] += __shfl_xor_sync(0xffffffffu, g[c], o);
+            }
+            if (lane == 0) {
+                s_loss[rg] = acc;
+#pragma unroll
+                for (int c = 0; c < 6; ++c) s_col[i & 1][rg][c] = g[c];
+            }
+        }
+        if (warp != 0) {
+            __syncwarp();
+            cluster_wait();
+            fence_after_sync();
+        }
+        if (TRAIN && i >= 3) {
+            __syncthreads();
+            if (i == 3 ? (rank == 0 && tid < 6) : tid < BN) {
+                float t = 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) t += s_col[i & 1][q][tid];
+                p.colpart[(long)tile * COLS + (i == 3 ? 768 : l * 256 + rank * BN) + tid] = t;
+                if (i == 3 && tid == 0) p.loss[tile] = (s_loss[0] + s_loss[1]) + (s_loss[2] + s_loss[3]);
+            }
+            __syncwarp();
         }
     }
     if (!ok) {
         atomicExch(p.status, 1);
         if (tid == 0) bar_wait(&full, (NPROD - 1) & 1);   // no copy outlives the CTA
     }
+    fence_before_sync();
     __syncthreads();
-    if (warp == 0) tmem_free(tmem, BN);
+    if (warp == 0) {
+        fence_after_sync();
+        tmem_free(tmem, BN);
+    }
 }
 
 }  // namespace

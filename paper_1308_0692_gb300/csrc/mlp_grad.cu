@@ -82,8 +82,9 @@ __global__ void __launch_bounds__(256, 1)
             }
             unsigned char *st = smem + s * STAGE;
             bar_expect(&full[s], (unsigned)((UM + t.n) * 128));
-            tma_load_2d(st, &maps.g[t.l], kt * UK, t.m0, &full[s]);
-            tma_load_2d(st + UM * 128, &maps.a[t.l], kt * UK, t.n0, &full[s]);
+            const int x = (kt & 1) * UK, z = kt >> 1;          // ROWS = 2 UK
+            tma_load_3d(st, &maps.g[t.l], x, t.m0, z, &full[s]);
+            tma_load_3d(st + UM * 128, &maps.a[t.l], x, t.n0, z, &full[s]);
         }
         // the copies still in flight land before the CTA can exit
         for (int j = issued > STAGES ? issued - STAGES : 0; j < issued; ++j) bar_wait(&full[j % STAGES], (j / STAGES) & 1);
@@ -200,16 +201,18 @@ __global__ void __launch_bounds__(256) mlp_reduce_adam_kernel(const __grid_const
     // sums with lane = row n (the partial tiles' order)
     float s[4] = {0.f, 0.f, 0.f, 0.f};
     const int n = n0 + lane;
+    if (n < nl) {
+        // the block's 32 columns lie in one partial tile; eight splits of loads in flight
+        const float *src = a.part + (long)tile_at(l, n, k0) * a.splits * (128 * 128) + ((k0 & 127) + w) * 128 + (n & 127);
+        const int nq = kl - k0 - w > 0 ? min(4, (kl - k0 - w + 7) / 8) : 0;
+#pragma unroll 8
+        for (int z = 0; z < a.splits; ++z)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int k = k0 + w + 8 * q;
-        if (n < nl && k < kl) {
-            const float *src = a.part + (long)tile_at(l, n, k) * a.splits * (128 * 128) + (k & 127) * 128 + (n & 127);
-#pragma unroll 4
-            for (int z = 0; z < a.splits; ++z) s[q] += src[(long)z * (128 * 128)];
-        }
-        tile[w + 8 * q][lane] = s[q];
+            for (int q = 0; q < 4; ++q)
+                if (q < nq) s[q] += src[(long)z * (128 * 128) + q * 8 * 128];
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tile[w + 8 * q][lane] = s[q];
     __syncthreads();
     // parameters with lane = column k
     const int k = k0 + lane;

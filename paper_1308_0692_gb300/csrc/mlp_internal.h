@@ -25,18 +25,17 @@ struct ChainArgs {
     const float *t;            // targets [M][6] (training)
     float *y;                  // [M][6] (inference)
     const float *b[NL];
-    // training: what the weight gradients need, transposed ([column][row], row pitch ld), and per
-    // row tile the bias gradients and the squared error
+    // training: what the weight gradients need, transposed ([tile][column][ROWS]), and per row
+    // tile the bias gradients and the squared error
     __nv_bfloat16 *aT[NL], *gT[NL];
-    float *gp;                 // GELU'(z) of the hidden layers [3][256][ld]
+    float *gp;                 // GELU'(z) of the hidden layers [tiles][3][256][ROWS]
     float *colpart;            // [tiles][COLS]
     double *loss;              // [tiles]
-    long ld;
     int M;
     int *status;
 };
 
-// tensor maps of the weight gradients: g_l^T and a_l^T
+// tensor maps of the weight gradients: g_l^T and a_l^T, three-dimensional (row of the tile, column, tile)
 struct GradMaps {
     CUtensorMap g[NL], a[NL];
 };

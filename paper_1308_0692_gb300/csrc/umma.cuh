@@ -55,6 +55,13 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
                  : "memory");
 }
 
+__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, int x, int y, int z, uint64_t *b)
+{
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n"
+                 ::"r"(su32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(su32(b))
+                 : "memory");
+}
+
 // Shared-memory matrix descriptor of a K-major tile with 128-byte swizzling: rows of 128 bytes,
 // 8-row groups 1024 bytes apart (stride byte offset), descriptor version 1, layout code 2.
 __device__ __forceinline__ uint64_t smem_desc(const void *tile)
@@ -144,18 +151,19 @@ inline EncodeTiled encoder()
     return fn;
 }
 
-// tensor map of a row-major BF16 matrix [rows][cols] (row pitch ld elements), box [box_rows][64],
-// rows and columns beyond the matrix filled with zeros
-inline bool make_map(CUtensorMap *map, const __nv_bfloat16 *base, int rows, long cols, long ld, int box_rows)
+// tensor map of BF16 matrices [slices][rows][cols], the rows ld elements apart, box
+// [1][box_rows][64], rows and columns beyond a matrix filled with zeros; slices = 0: one matrix,
+// a two-dimensional map
+inline bool make_map(CUtensorMap *map, const __nv_bfloat16 *base, int rows, int cols, int ld, int box_rows, int slices = 0)
 {
     EncodeTiled enc = encoder();
     if (!enc) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)UK, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16 *>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+    const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)(slices > 0 ? slices : 1)};
+    const cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)ld * 2 * rows};
+    const cuuint32_t box[3] = {(cuuint32_t)UK, (cuuint32_t)box_rows, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, slices > 0 ? 3 : 2, const_cast<__nv_bfloat16 *>(base), dims, strides, box,
+               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
