@@ -1016,35 +1016,262 @@ __global__ void __launch_bounds__(256, G == M ? 3 : (2 * G == M ? 2 : 1)) batch_
     }
 }
 
-// six linearised moments of one instance (rho, ux, uy, pxx, pxy, pyy per cell), FP64
-template <typename T>
-__global__ void inst_moments_kernel(const T *h, const BatchInst I, int m, const BatchArgs a, double u_ref, double *out)
+// Channels of one periodic column (Couette, nx = 1): one block marches an instance through all
+// the launch's steps with its state on chip -- two threads a cell, one for the velocity rows
+// that move down (iy < M / 2), one for those that move up, own values in registers.  After the
+// relaxation every thread puts its values into shared memory, from where the next cell takes
+// its upwind neighbours; the wall cells put Eq. 8's ghosts at the ends.  Two block barriers a
+// step (values published; neighbours read, which also carries the partial moments), no grid
+// barrier and no global traffic between steps: in the segment kernel's grid-wide barriers twelve channels
+// took 11 us a step.  Bound by a block's issue rate and shared-memory traffic, so a
+// channel takes the same time whether one or a hundred others run beside it.  (Neighbours by
+// warp shuffles with the warps' edges through shared memory, one thread a cell, took 7.2 us a
+// step for 500 cells.)  The arithmetic is batch_group's, the sums of the wall density across velocity
+// rows compensated FP32 (comp_add) instead of FP64, as in the column march of the cavities.
+// On residual steps the old state passes through the instance's buffer of that step.
+constexpr int COLUMN_CELLS = 512;
+
+template <int M>
+struct ColumnShared {
+    static constexpr int NP = M * M / 4;                 // velocity pairs of a thread: half the rows
+    float2 v[2][NP][COLUMN_CELLS + 1];                   // down: cell c at c, the top ghosts at ny; up: c at c + 1, the bottom ghosts at 0
+    float4 mom[2][COLUMN_CELLS];
+    double sum[2][32];
+    int stop;
+};
+
+template <int M, int MODE>
+__global__ void __launch_bounds__(2 * COLUMN_CELLS, 1) batch_column_kernel(const BatchArgs a, const int *list)
 {
-    const long ncells = I.ncells;
-    for (long c = (long)blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += (long)gridDim.x * blockDim.x) {
-        const int yc = (int)(c / I.nx), xc = (int)(c - (long)yc * I.nx);
-        double s0 = 0, sx = 0, sy = 0, sxx = 0, sxy = 0, syy = 0;
-        for (int iy = 0; iy < m; ++iy) {
-            const double ey = a.xi[iy];
-            for (int ix = 0; ix < m; ++ix) {
-                const double ex = a.xi[ix];
-                const double v = (double)h[inst_index(I, m * m, iy * m + ix, xc, yc)];
-                s0 += v;
-                sx += ex * v;
-                sy += ey * v;
-                sxx += ex * ex * v;
-                sxy += ex * ey * v;
-                syy += ey * ey * v;
+    using Sh = ColumnShared<M>;
+    constexpr int P = M / 2, HALF = M / 2, NP = Sh::NP;
+    extern __shared__ __align__(16) unsigned char column_smem[];
+    Sh &sh = *reinterpret_cast<Sh *>(column_smem);
+    const int inst = list[blockIdx.x];
+    if (a.frozen[inst] <= a.step0) return;
+    const BatchInst &I = a.inst[inst];
+    const int ny = I.ny, width = blockDim.x / 2;         // width: whole warps
+    const int up = threadIdx.x >= width, cell = threadIdx.x - up * width;
+    const bool on = cell < ny;
+    const int r0 = up * HALF;
+    const float cy = (float)I.cy, om = (float)I.omega, bb = (float)I.b;
+    float xiy[HALF], wy[HALF];
+#pragma unroll
+    for (int r = 0; r < HALF; ++r) {
+        xiy[r] = a.xi_f[r0 + r];
+        wy[r] = a.w1_f[r0 + r];
+    }
+    // the wall this thread's rows leave through gives ghosts to the other rows (Eq. 8)
+    const float uw = (float)(up ? I.u_top : I.u_bottom);
+    const float drive = MODE == BATCH_CORRECT ? 0.f : (float)((up ? I.u_top : I.u_bottom) * I.inv_u_ref);
+    const bool at_wall = on && cell == (up ? ny - 1 : 0);
+    float2 *const ghost = &sh.v[up ^ 1][0][up ? ny : 0], *const mine = &sh.v[up][0][cell + up];
+    const float2 *const upwind = &sh.v[up][0][up ? cell : cell + 1];
+    constexpr int PITCH = COLUMN_CELLS + 1;
+    auto base = [&](long s) { return static_cast<float *>(a.buf[s & 1]) + I.off + (long)r0 * M * ny + cell; };
+    float2 h[NP];
+    {
+        const float *src = base(a.step0);
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+            h[q] = on ? make_float2(src[(long)(2 * q) * ny], src[(long)(2 * q + 1) * ny]) : make_float2(0.f, 0.f);
+    }
+    long s = a.step0;
+    const long end = a.step0 + a.nsteps;
+    while (s < end) {
+        const bool resid = (s + 1) % a.resid_every == 0;
+        // publish the values and, at the wall, the ghosts
+        if (on)
+#pragma unroll
+            for (int q = 0; q < NP; ++q) mine[q * PITCH] = h[q];
+        if (at_wall) {                                   // Eq. 9: what these rows carry into the wall
+            float hi = 0.f, lo = 0.f;
+#pragma unroll
+            for (int r = 0; r < HALF; ++r) {
+                float sum = 0.f;
+#pragma unroll
+                for (int j = 0; j < P; ++j) {
+                    sum += h[r * P + j].x;
+                    sum += h[r * P + j].y;
+                }
+                const float ax = fabsf(xiy[r]), p = ax * sum;
+                comp_add(hi, lo, p);
+                lo += fmaf(ax, sum, -p);
+            }
+            const float rho = fmaf(hi, a.inv_dy_wall_f, lo * a.inv_dy_wall_f);
+#pragma unroll
+            for (int r = 0; r < HALF; ++r)
+#pragma unroll
+                for (int j = 0; j < P; ++j) {
+                    const float2 wa = __fmul2_rn(w2(a, j), splat(a.w1_f[HALF - r0 + r]));
+                    const float2 gg = __ffma2_rn(xi2(a, j), splat(uw), splat(1.f));
+                    ghost[(r * P + j) * PITCH] = __fmul2_rn(wa, __ffma2_rn(xi2(a, j), splat(drive), __fmul2_rn(splat(rho), gg)));
+                }
+        }
+        __syncthreads();
+        if (resid && on) {
+            float *at = base(s);
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                at[(long)(2 * q) * ny] = h[q].x;
+                at[(long)(2 * q + 1) * ny] = h[q].y;
             }
         }
-        const double rho = 1.0 + u_ref * s0;
-        out[c] = rho;
-        out[ncells + c] = u_ref * sx / rho;
-        out[2 * ncells + c] = u_ref * sy / rho;
-        out[3 * ncells + c] = 1.0 + u_ref * sxx;
-        out[4 * ncells + c] = u_ref * sxy;
-        out[5 * ncells + c] = 1.0 + u_ref * syy;
+        float rho = 0.f, jx = 0.f, jy = 0.f;
+#pragma unroll
+        for (int r = 0; r < HALF; ++r) {
+            const float2 nuy = splat(fabsf(xiy[r]) * cy);
+            float2 R2 = make_float2(0.f, 0.f), X2 = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < P; ++j) {
+                const int q = r * P + j;
+                const float2 hn = upwind[q * PITCH];
+                const float2 t = __ffma2_rn(nuy, __fadd2_rn(hn, neg2(h[q])), h[q]);
+                h[q] = t;
+                R2 = __fadd2_rn(R2, t);
+                X2 = __ffma2_rn(xi2(a, j), t, X2);
+            }
+            const float R = R2.x + R2.y;
+            rho += R;
+            jx += X2.x + X2.y;
+            jy += xiy[r] * R;
+        }
+        sh.mom[up][cell] = make_float4(rho, jx, jy, 0.f);
+        __syncthreads();
+        {
+            const float4 m0 = sh.mom[0][cell], m1 = sh.mom[1][cell];
+            rho = m0.x + m1.x;
+            jx = m0.y + m1.y;
+            jy = m0.z + m1.z;
+        }
+        double sd = 0.0, sn = 0.0;
+        const float *src = MODE == BATCH_CORRECT ? a.src + I.off + (long)r0 * M * ny + cell : nullptr;
+#pragma unroll
+        for (int r = 0; r < HALF; ++r) {
+            const float wom = om * wy[r];
+            const float2 qv = splat(wom * (rho + xiy[r] * jy)), jj = splat(wom * jx);
+#pragma unroll
+            for (int j = 0; j < P; ++j) {
+                const int q = r * P + j;
+                float2 v = __ffma2_rn(w2(a, j), __ffma2_rn(xi2(a, j), jj, qv), __fmul2_rn(splat(bb), h[q]));
+                if (MODE == BATCH_CORRECT && on)
+                    v = __fadd2_rn(v, make_float2(src[(long)(2 * q) * ny], src[(long)(2 * q + 1) * ny]));
+                h[q] = v;
+            }
+        }
+        if (resid) {
+            const float *old = base(s);
+            if (on)
+#pragma unroll
+                for (int r = 0; r < HALF; ++r) {
+                    float2 d2 = make_float2(0.f, 0.f), n2 = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int j = 0; j < P; ++j) {
+                        const int q = r * P + j;
+                        const float2 d = __fadd2_rn(h[q], neg2(make_float2(old[(long)(2 * q) * ny], old[(long)(2 * q + 1) * ny])));
+                        d2 = __ffma2_rn(d, d, d2);
+                        n2 = __ffma2_rn(h[q], h[q], n2);
+                    }
+                    sd += (double)(d2.x + d2.y);
+                    sn += (double)(n2.x + n2.y);
+                }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sd += __shfl_xor_sync(0xffffffffu, sd, o);
+                sn += __shfl_xor_sync(0xffffffffu, sn, o);
+            }
+            if ((threadIdx.x & 31) == 0) {
+                sh.sum[0][threadIdx.x >> 5] = sd;
+                sh.sum[1][threadIdx.x >> 5] = sn;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                double d = 0.0, n = 0.0;
+                for (int w = 0; w < (int)blockDim.x / 32; ++w) {
+                    d += sh.sum[0][w];
+                    n += sh.sum[1][w];
+                }
+                a.acc[2 * inst] = d;
+                a.acc[2 * inst + 1] = n;
+                residual_decision<MODE>(a, inst, s);
+                sh.stop = a.frozen[inst] <= s + 1;
+            }
+            __syncthreads();
+        }
+        ++s;
+        if (resid && sh.stop) break;
     }
+    if (on) {
+        float *at = base(s);
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            at[(long)(2 * q) * ny] = h[q].x;
+            at[(long)(2 * q + 1) * ny] = h[q].y;
+        }
+    }
+}
+
+// The state an instance stands at: frozen (at its convergence step) or at the batch's step.
+// Six linearised moments (rho, ux, uy, pxx, pxy, pyy per cell), FP64: a block takes 32 cells,
+// warp w velocity row w, whose sums over pairs of opposite velocities cost three and a half
+// FP64 operations per velocity (conversion included); then warp k < 6 forms output k from the
+// M row sums.  As one thread per cell with nine FP64 operations per velocity a 128^2 cavity
+// took 48 us, bound by the FP64 pipe and one thread's chain.
+template <int M>
+__global__ void __launch_bounds__(32 * (M > 6 ? M : 6))
+    inst_moments_kernel(const float *b0, const float *b1, const long *frozen, long step, const BatchInst I, const BatchArgs a,
+                        double u_ref, double *out)
+{
+    __shared__ double s[3][M][32];          // row sums of v, xi_x v, xi_x^2 v
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long f = *frozen, at = f == LONG_MAX ? step : f;
+    const float *h = ((at & 1) ? b1 : b0) + I.off;
+    long c;
+    int x, y;
+    bool on;
+    if (I.tiled) {
+        const int tiles = (I.nx + 31) >> 5;
+        y = (int)(blockIdx.x / tiles);
+        x = (int)(blockIdx.x % tiles) * 32 + lane;
+        on = x < I.nx;
+        c = (long)y * I.nx + x;
+        if (!on) x = I.nx - 1;
+    } else {
+        c = (long)blockIdx.x * 32 + lane;
+        on = c < I.ncells;
+        const long cc = on ? c : I.ncells - 1;
+        y = (int)(cc / I.nx);
+        x = (int)(cc % I.nx);
+    }
+    if (w < M) {
+        double S = 0.0, X = 0.0, XX = 0.0;
+#pragma unroll
+        for (int ix = 0; ix < M / 2; ++ix) {         // xi[M-1-ix] = -xi[ix]
+            const double p = (double)h[inst_index(I, M * M, w * M + M - 1 - ix, x, y)];
+            const double n = (double)h[inst_index(I, M * M, w * M + ix, x, y)];
+            const double sum = p + n, dif = p - n, e = a.xi[M - 1 - ix];
+            S += sum;
+            X += e * dif;
+            XX += (e * e) * sum;
+        }
+        s[0][w][lane] = S;
+        s[1][w][lane] = X;
+        s[2][w][lane] = XX;
+    }
+    __syncthreads();
+    if (w >= 6 || !on) return;
+    double v = 0.0, rho = 0.0;
+    const int k = w == 1 || w == 4 ? 1 : w == 3 ? 2 : 0;
+#pragma unroll
+    for (int r = 0; r < M; ++r) {
+        const double e = a.xi[r];
+        if (w <= 2) rho += s[0][r][lane];
+        if (w == 1 || w == 3) v += s[k][r][lane];
+        if (w == 2 || w == 4) v += e * s[k][r][lane];
+        if (w == 5) v += (e * e) * s[0][r][lane];
+    }
+    rho = 1.0 + u_ref * rho;
+    out[w * I.ncells + c] = w == 0 ? rho : w <= 2 ? u_ref * v / rho : w == 4 ? u_ref * v : 1.0 + u_ref * v;
 }
 
 template <typename TS, typename TC, int M, int G, int MODE>
@@ -1141,7 +1368,9 @@ struct lbm_batch {
     BatchInst *d_inst;
     BatchItem *d_items;
     MarchItem *d_mitems;        // column-march items (cavity instances when the march is on)
-    unsigned char *d_kind;      // [count] 1: cavity instance marched by columns
+    int *d_cols;                // one-column channels marched by batch_column_kernel
+    unsigned char *d_kind;      // [count] 0: by segments, 1: cavity marched by columns, 2: one-column channel
+    int ncols, col_threads;     // their number, threads of a block (two a cell, whole warps)
     bool march;                 // cavity instances by the column-march kernel
     int nmitems, mgrid, mchunk; // march items, their co-resident grid, rows per chunk
     std::vector<int> iitems;    // march items per instance (host copy of d_iitems)
@@ -1253,7 +1482,15 @@ BatchItem make_item(const BatchInst &I, int inst, int seg)
     return t;
 }
 
-bool marched(const lbm_batch *b, int i, bool march) { return march && b->inst[i].cavity; }
+// channels batch_column_kernel takes: one periodic column that fits a block
+bool column_channel(const lbm_batch *b, int i)
+{
+    const BatchInst &I = b->inst[i];
+    return !I.cavity && I.nx == 1 && I.ny <= COLUMN_CELLS;
+}
+
+bool marched(const lbm_batch *b, int i, bool march) { return march && (b->inst[i].cavity || column_channel(b, i)); }
+unsigned char kind_of(const lbm_batch *b, int i) { return !marched(b, i, b->march) ? 0 : b->inst[i].cavity ? 1 : 2; }
 
 void build_items(const lbm_batch *b, int order, bool march, std::vector<BatchItem> &bulk, std::vector<BatchItem> &wall)
 {
@@ -1408,9 +1645,27 @@ lbm_status apply_schedule_march(lbm_batch *b, int g, int bpsm, int order, bool m
         build_march_items(b, rows, mitems);
         mgrid = (int)std::min<long>((long)nsm * mb, std::max<long>(1, ((long)mitems.size() + sub - 1) / sub));
     }
+    std::vector<int> cols;
+    int col_threads = 64;
+    for (int i = 0; i < (int)b->inst.size(); ++i)
+        if (march && b->live[i] && column_channel(b, i)) {
+            cols.push_back(i);
+            col_threads = std::max(col_threads, (b->inst[i].ny + 31) / 32 * 64);
+        }
+    if (!cols.empty()) {
+        const size_t smem = b->m == 8 ? sizeof(ColumnShared<8>) : sizeof(ColumnShared<4>);
+        void *fn[2] = {b->m == 8 ? (void *)batch_column_kernel<8, BATCH_MARCH> : (void *)batch_column_kernel<4, BATCH_MARCH>,
+                       b->m == 8 ? (void *)batch_column_kernel<8, BATCH_CORRECT> : (void *)batch_column_kernel<4, BATCH_CORRECT>};
+        for (void *f : fn) {
+            e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return bfail(LBM_ECUDA, std::string("one-column channel kernel: ") + cudaGetErrorString(e));
+        }
+    }
     // stream-ordered uploads (pageable sources are staged before the calls return)
     e = cudaSuccess;
-    if (!mitems.empty()) {
+    if (!cols.empty())
+        e = cudaMemcpyAsync(b->d_cols, cols.data(), sizeof(int) * cols.size(), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess && !mitems.empty()) {
         b->iitems.assign(b->inst.size(), 0);
         for (const MarchItem &t : mitems) b->iitems[t.inst] += 1;
         e = cudaMemcpyAsync(b->d_mitems, mitems.data(), sizeof(MarchItem) * mitems.size(), cudaMemcpyHostToDevice,
@@ -1437,6 +1692,8 @@ lbm_status apply_schedule_march(lbm_batch *b, int g, int bpsm, int order, bool m
     b->nmitems = (int)mitems.size();
     b->mgrid = mgrid;
     b->mchunk = mchunk;
+    b->ncols = (int)cols.size();
+    b->col_threads = col_threads;
     const int spb = segs_per_block(g);
     const long groups = std::max(((long)b->nitems + spb - 1) / spb, ((long)b->nwall + spb - 1) / spb);
     b->grid = (int)std::min<long>((long)nsm * bpsm, std::max<long>(1, groups));
@@ -1513,17 +1770,29 @@ cudaError_t launch_coop(void *fn, int grid, int threads, const BatchArgs &a, cud
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-// One advance: the column-march kernel over the cavity items, then the segment kernel over
-// the other instances' items (each launched only when it has items).
-cudaError_t launch_pair(lbm_batch *b, const BatchArgs &a0, void *mfn, void *sfn, cudaStream_t st)
+// One advance: the one-column channels, the column-march kernel over the cavity items, then the
+// segment kernel over the other instances' items (each launched only when it has some).
+cudaError_t launch_all(lbm_batch *b, const BatchArgs &a0, bool correct, cudaStream_t st)
 {
+    const MarchFns mf = march_fns(b->m, b->mg);
+    void *mfn = correct ? mf.correct : mf.march, *sfn = correct ? b->var->fn_correct : b->var->fn;
     cudaError_t e = cudaSuccess;
+    if (b->ncols > 0) {
+        if (b->m == 8)
+            correct ? batch_column_kernel<8, BATCH_CORRECT><<<b->ncols, b->col_threads, sizeof(ColumnShared<8>), st>>>(a0, b->d_cols)
+                    : batch_column_kernel<8, BATCH_MARCH><<<b->ncols, b->col_threads, sizeof(ColumnShared<8>), st>>>(a0, b->d_cols);
+        else
+            correct ? batch_column_kernel<4, BATCH_CORRECT><<<b->ncols, b->col_threads, sizeof(ColumnShared<4>), st>>>(a0, b->d_cols)
+                    : batch_column_kernel<4, BATCH_MARCH><<<b->ncols, b->col_threads, sizeof(ColumnShared<4>), st>>>(a0, b->d_cols);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     if (b->nmitems > 0) {
         BatchArgs a = a0;
         a.kind_sel = 1;
         e = cudaMemsetAsync(a.mcount, 0, 2 * sizeof(unsigned), st);
         if (e == cudaSuccess) e = cudaMemsetAsync(a.ifin, 0, 2 * sizeof(unsigned) * b->inst.size(), st);
-        if (e == cudaSuccess) e = launch_coop(mfn, b->mgrid, 256, a, st, march_fns(b->m, b->mg).smem);
+        if (e == cudaSuccess) e = launch_coop(mfn, b->mgrid, 256, a, st, mf.smem);
     }
     if (e == cudaSuccess && (b->nitems > 0 || b->nwall > 0)) {
         BatchArgs a = a0;
@@ -1533,10 +1802,7 @@ cudaError_t launch_pair(lbm_batch *b, const BatchArgs &a0, void *mfn, void *sfn,
     return e;
 }
 
-cudaError_t launch_batch(lbm_batch *b, const BatchArgs &a, cudaStream_t st)
-{
-    return launch_pair(b, a, march_fns(b->m, b->mg).march, b->var->fn, st);
-}
+cudaError_t launch_batch(lbm_batch *b, const BatchArgs &a, cudaStream_t st) { return launch_all(b, a, false, st); }
 
 // Co-resident grid of a kernel of this batch for the current item lists.
 int coop_grid(lbm_batch *b, void *fn, int threads, int g)
@@ -1679,6 +1945,7 @@ static lbm_status batch_layout(const lbm_vset *vs, const lbm_problem *insts, int
     off = align256(off + sizeof(BatchInst) * count);
     off = align256(off + sizeof(BatchItem) * segs);
     off = align256(off + sizeof(MarchItem) * std::max(1L, mits));
+    off = align256(off + sizeof(int) * count);                  // one-column channels
     off = align256(off + (size_t)count);                        // instance kinds
     off = align256(off + sizeof(double) * 2 * count);
     off = align256(off + sizeof(double) * count);     // last residual
@@ -1756,7 +2023,8 @@ lbm_status lbm_batch_init(const lbm_vset *vs, const lbm_problem *insts, int coun
     b->timeout_cycles = 4000000000LL;   // about 2 s at the GB300 SM clock
     b->ref_base = nullptr;
     b->march = march_fns(m).march != nullptr;
-    b->nmitems = b->mgrid = b->mchunk = 0;
+    b->nmitems = b->mgrid = b->mchunk = b->ncols = 0;
+    b->col_threads = 64;
     b->nsm = 0;
     b->mchunk_fixed = 0;
     b->mg = 0;
@@ -1782,6 +2050,8 @@ lbm_status lbm_batch_init(const lbm_vset *vs, const lbm_problem *insts, int coun
     o = align256(o + sizeof(BatchItem) * segs);
     b->d_mitems = (MarchItem *)(p + o);
     o = align256(o + sizeof(MarchItem) * std::max(1L, mits));
+    b->d_cols = (int *)(p + o);
+    o = align256(o + sizeof(int) * count);
     b->d_kind = (unsigned char *)(p + o);
     o = align256(o + (size_t)count);
     b->d_acc = (double *)(p + o);
@@ -1816,7 +2086,7 @@ lbm_status lbm_batch_init(const lbm_vset *vs, const lbm_problem *insts, int coun
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_frozen, frozen.data(), sizeof(long) * count, cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_bar, 0, 64, b->stream);
     std::vector<unsigned char> kind(count);
-    for (int i = 0; i < count; ++i) kind[i] = marched(b, i, b->march) ? 1 : 0;
+    for (int i = 0; i < count; ++i) kind[i] = kind_of(b, i);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_kind, kind.data(), count, cudaMemcpyHostToDevice, b->stream);
     std::vector<double> tab(2 * LBM_MAX_M, 0.0);
     for (int k = 0; k < m; ++k) {
@@ -1869,7 +2139,7 @@ lbm_status lbm_batch_set_march(lbm_batch *b, int on, int rows_per_chunk, int war
     b->mg = warps_per_item;
     const int n = (int)b->inst.size();
     std::vector<unsigned char> kind(n);
-    for (int i = 0; i < n; ++i) kind[i] = marched(b, i, b->march) ? 1 : 0;
+    for (int i = 0; i < n; ++i) kind[i] = kind_of(b, i);
     cudaError_t e = cudaMemcpyAsync(b->d_kind, kind.data(), n, cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bfail(LBM_ECUDA, std::string("setting the march: ") + cudaGetErrorString(e));
@@ -2100,14 +2370,14 @@ lbm_status lbm_batch_moments(lbm_batch *b, int i, double *out_dev)
 {
     if (!b || !out_dev) return bfail(LBM_EINVAL, "NULL argument");
     if (i < 0 || i >= (int)b->inst.size()) return bfail(LBM_EINVAL, "instance index out of range");
-    long steps;
-    lbm_status st = lbm_batch_status(b, i, &steps, nullptr, nullptr);
-    if (st != LBM_OK) return st;
     const BatchArgs a = make_args(b, 1, 0.0);
     const BatchInst &I = b->inst[i];
-    const int nb = (int)std::min<long>(1216, (I.ncells + 255) / 256);
-    const float *h = (const float *)b->buf[steps & 1] + I.off;
-    inst_moments_kernel<float><<<nb, 256, 0, b->stream>>>(h, I, b->m, a, 1.0 / I.inv_u_ref, out_dev);
+    const long blocks = I.tiled ? (long)((I.nx + 31) / 32) * I.ny : (I.ncells + 31) / 32;
+    const float *b0 = (const float *)b->buf[0], *b1 = (const float *)b->buf[1];
+    if (b->m == 8)
+        inst_moments_kernel<8><<<(unsigned)blocks, 256, 0, b->stream>>>(b0, b1, b->d_frozen + i, b->step, I, a, 1.0 / I.inv_u_ref, out_dev);
+    else
+        inst_moments_kernel<4><<<(unsigned)blocks, 192, 0, b->stream>>>(b0, b1, b->d_frozen + i, b->step, I, a, 1.0 / I.inv_u_ref, out_dev);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LBM_OK : bfail(LBM_ECUDA, std::string("instance moments: ") + cudaGetErrorString(e));
 }
@@ -2243,7 +2513,7 @@ lbm_status lbm_batch_refine(lbm_batch *b, double tol, int max_sweeps, double ref
     a.flat = nullptr;
             a.frozen = b->r_frozen;
             a.step0 = k;
-            e = launch_pair(b, a, march_fns(b->m, b->mg).correct, b->var->fn_correct, b->stream);
+            e = launch_all(b, a, true, b->stream);
             k += chunk;
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(fro.data(), b->r_frozen, sizeof(long) * n, cudaMemcpyDeviceToHost, b->stream);
