@@ -334,7 +334,20 @@ cudaError_t commit_planar(lbm_sim *s)
                                s->prob.ny, s->tile_pitch, s->stream);
 }
 
-StepArgs base_args(const lbm_sim *s) { return s->args; }
+// FP64 tables of step_tile.cuh for the relaxation factors in `a`: with b = 1 - omega folded into
+// the transport, relaxing costs two operations per velocity instead of two and a half.  The
+// moments then come out times b, so a small b (dt near Kn) stays outside.
+void scale_tables(StepArgs &a, int m)
+{
+    a.fold = a.b >= 0.0625;
+    const double s = a.fold ? a.b : 1.0;
+    for (int i = 0; i < m; ++i) {
+        a.nux_s[i] = s * a.nux[i];
+        a.nuy_s[i] = s * a.nuy[i];
+        a.omw[i] = a.omega / s * a.w1[i];
+        for (int k = 0; k < m; ++k) a.a0[i * m + k] = s * (1.0 - a.nux[k] - a.nuy[i]);
+    }
+}
 
 void fill_args(lbm_sim *s, const TableHeader &hdr)
 {
@@ -377,10 +390,9 @@ void fill_args(lbm_sim *s, const TableHeader &hdr)
             a.so_c_f[ax][i] = (float)a.so_c[ax][i];
         }
     }
-    for (int iy = 0; iy < v.m; ++iy)
-        for (int ix = 0; ix < v.m; ++ix) a.a0[iy * v.m + ix] = 1.0 - a.nux[ix] - a.nuy[iy];
     a.omega = s->omega;
     a.b = 1.0 - s->omega;
+    scale_tables(a, v.m);
     a.omega_f = (float)a.omega;
     a.b_f = (float)a.b;
     a.inv_dx_wall = hdr.inv_dx_wall;
@@ -1178,6 +1190,7 @@ lbm_status lbm_set_splitting(lbm_sim *s, int scheme)
     s->args.omega = 1.0 - b;
     s->args.b_f = (float)b;
     s->args.omega_f = (float)(1.0 - b);
+    scale_tables(s->args, s->vs.m);
     drop_graphs(s);
     return LBM_OK;
 }

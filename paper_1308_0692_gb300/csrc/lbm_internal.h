@@ -80,7 +80,10 @@ struct StepArgs {
     double nuy[LBM_MAX_M];  // |xi| dt / dy
     double w1[LBM_MAX_M];   // 1-D weights (w_a = w1[ix] w1[iy])
     double wxi[LBM_MAX_M];  // w1 xi
-    double a0[LBM_MAX_V];   // 1 - nux[ix] - nuy[iy]
+    // FP64 form of step_tile.cuh, scaled by s = 1 - omega (fold) or 1: transport coefficients
+    // s (1 - nux - nuy), s nux, s nuy, and (omega / s) w1
+    double a0[LBM_MAX_V], nux_s[LBM_MAX_M], nuy_s[LBM_MAX_M], omw[LBM_MAX_M];
+    int fold;
     float xi_f[LBM_MAX_M], nux_f[LBM_MAX_M], nuy_f[LBM_MAX_M], w1_f[LBM_MAX_M];
     // second-order transport, per axis (0: x, 1: y) and node with Courant number nu:
     // P = nu (3 - nu) / 2, B = nu (2 - nu), and the second upwind cell's coefficient

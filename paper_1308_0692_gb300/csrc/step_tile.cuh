@@ -19,9 +19,11 @@
 // that puts Eq. 8's ghost in the upwind place.
 //
 // FP64 arithmetic.  GB300 retires about two FP64 lanes per cycle and SM, so the FP64 form
-// counts its operations: transport as (1 - nu_x - nu_y) h + nu_x h_x + nu_y h_y (three, the
-// first coefficient a host table), two for the moment sums, two and a half for the relaxation
-// (the opposite velocities ix and M-1-ix share w_x q: w_x q +- w_x xi_x J).  The FP32 form
+// counts its operations, seven per velocity and a few per row: transport as
+// s [(1 - nu_x - nu_y) h + nu_x h_x + nu_y h_y] with s = 1 - omega (three, the coefficients host
+// tables), two for the moment sums, two for the relaxation, which only adds
+// w_x q + w_x xi_x J to the scaled transported value.  (Where 1 - omega is below 1/16, s = 1 and
+// the factor is applied after the moments.)  The FP32 form
 // keeps h + nu_x (h_x - h) + nu_y (h_y - h), which moves a constant state without rounding.
 #pragma once
 
@@ -46,7 +48,7 @@ __global__ void __launch_bounds__(tile_cells<NS>() * NS) step_tile_kernel(const 
     __shared__ TC s_mom[3][NS][CELLS];
     __shared__ double s_wall[4][NS][CELLS];
     __shared__ TC s_tot[TWO ? 3 : 1][CELLS];
-    __shared__ double s_red[2][ACC ? CELLS * NS : 1];
+    __shared__ double s_red[2][(CELLS * NS + 31) / 32];
 
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int W = blockDim.x, g = threadIdx.y;
@@ -133,35 +135,36 @@ __global__ void __launch_bounds__(tile_cells<NS>() * NS) step_tile_kernel(const 
 
     // ---- transport (upwind) + moment sums, transported values in registers ----
     TC rho = 0, jx = 0, jy = 0;
-    auto transport = [&](auto walls_tag) {
-        constexpr bool WALLS = decltype(walls_tag)::value;
+    auto transport = [&](auto xwalls_tag, auto ywalls_tag) {
+        constexpr bool XW = decltype(xwalls_tag)::value, YW = decltype(ywalls_tag)::value;
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
             const int iy = g * RPL + r;
             const bool ypos = iy >= M - HALF, yneg = iy < HALF;
             const long dy = ypos ? dn : (yneg ? up : 0);
-            const TC nuy = pick<TC>(a.nuy, a.nuy_f, iy), wy = pick<TC>(a.w1, a.w1_f, iy);
-            const bool ywall = WALLS && ((ypos && wb) || (yneg && wt));
+            const TC nuy = pick<TC>(a.nuy_s, a.nuy_f, iy), wy = pick<TC>(a.w1, a.w1_f, iy);
+            const bool ywall = YW && ((ypos && wb) || (yneg && wt));
             TC gy0 = 0, gy1 = 0;                       // ghost w_x (gy0 + xi_x gy1) of a y wall
-            if (WALLS) {
+            if (YW) {
                 const TC d = ypos ? rb : rt, u = (TC)(ypos ? a.u_bottom : a.u_top);
                 const TC drive = a.homogeneous ? TC(0) : (TC)((ypos ? a.u_bottom : a.u_top) * a.inv_u_ref);
                 gy0 = wy * d;
                 gy1 = wy * (d * u + drive);
             }
-            TC R = 0, X = 0;
+            TC R = 0;
+            [[maybe_unused]] TC X = 0;                 // FP32: the row's sum first
 #pragma unroll
             for (int ix = 0; ix < M; ++ix) {
                 const TS *hv = hp + (long)(r * M + ix) * ncells;
                 const TC hc = hs[r * M + ix], xix = pick<TC>(a.xi, a.xi_f, ix), wx = pick<TC>(a.w1, a.w1_f, ix);
                 TC hx = hc, hy = (TC)hv[dy];
-                if (ix >= M - HALF) hx = (WALLS && wl) ? wx * (wy * rl) : (TC)hv[dl];
-                else if (ix < HALF) hx = (WALLS && wr) ? wx * (wy * rr) : (TC)hv[dr];
-                if (WALLS && ywall) hy = wx * (gy0 + xix * gy1);
+                if (ix >= M - HALF) hx = (XW && wl) ? wx * (wy * rl) : (TC)hv[dl];
+                else if (ix < HALF) hx = (XW && wr) ? wx * (wy * rr) : (TC)hv[dr];
+                if (YW && ywall) hy = wx * (gy0 + xix * gy1);
                 TC v;
                 if constexpr (DP) {
                     v = a.a0[iy * M + ix] * hc;
-                    if (ix >= M - HALF || ix < HALF) v += a.nux[ix] * hx;
+                    if (ix >= M - HALF || ix < HALF) v += a.nux_s[ix] * hx;
                     v += nuy * hy;
                 } else {
                     v = hc;
@@ -170,15 +173,17 @@ __global__ void __launch_bounds__(tile_cells<NS>() * NS) step_tile_kernel(const 
                 }
                 hs[r * M + ix] = v;
                 R += v;
-                X += xix * v;
+                if constexpr (DP) jx += xix * v;
+                else X += xix * v;
             }
             rho += R;
-            jx += X;
+            if constexpr (!DP) jx += X;
             jy += pick<TC>(a.xi, a.xi_f, iy) * R;
         }
     };
-    if (walls) transport(std::true_type{});
-    else transport(std::false_type{});
+    if (!walls) transport(std::false_type{}, std::false_type{});
+    else if (__any_sync(__activemask(), wb || wt)) transport(std::true_type{}, std::true_type{});
+    else transport(std::true_type{}, std::false_type{});
     if (NS > 1) {
         s_mom[0][g][cl] = rho;
         s_mom[1][g][cl] = jx;
@@ -208,13 +213,15 @@ __global__ void __launch_bounds__(tile_cells<NS>() * NS) step_tile_kernel(const 
 
     // ---- relaxation, store, residual ----
     TC psd = 0, psn = 0;
-    const TC b = pick<TC>(&a.b, &a.b_f, 0), om = pick<TC>(&a.omega, &a.omega_f, 0);
+    if (DP && !a.fold)
+#pragma unroll
+        for (int k = 0; k < RPL * M; ++k) hs[k] *= (TC)a.b;
     TS *hn = reinterpret_cast<TS *>(a.hn) + (long)(g * RPL * M) * ncells + c;
     const TS *hsrc = SOURCE ? reinterpret_cast<const TS *>(a.src) + (long)(g * RPL * M) * ncells + c : nullptr;
 #pragma unroll
     for (int r = 0; r < RPL; ++r) {
         const int iy = g * RPL + r;
-        const TC wom = om * pick<TC>(a.w1, a.w1_f, iy);
+        const TC wom = DP ? (TC)a.omw[iy] : (TC)(a.omega_f * a.w1_f[iy]);
         const TC q = wom * (rho + pick<TC>(a.xi, a.xi_f, iy) * jy);
         const TC jj = wom * jx;
         auto put = [&](int ix, TC v) {
@@ -230,36 +237,40 @@ __global__ void __launch_bounds__(tile_cells<NS>() * NS) step_tile_kernel(const 
         };
         if constexpr (DP) {
 #pragma unroll
-            for (int ix = 0; ix < HALF; ++ix) {       // xi[M-1-ix] = -xi[ix], the same weight
-                const TC A = a.w1[ix] * q, wx = a.wxi[ix];
-                put(ix, b * hs[r * M + ix] + (wx * jj + A));
-                put(M - 1 - ix, b * hs[r * M + M - 1 - ix] + (A - wx * jj));
+            for (int ix = 0; ix < M; ++ix) {
+                TC v = a.w1[ix] * q + hs[r * M + ix];
+                if (2 * ix + 1 != M) v += a.wxi[ix] * jj;      // xi = 0 in the middle of an odd set
+                put(ix, v);
             }
-            if (M & 1) put(HALF, b * hs[r * M + HALF] + a.w1[HALF] * q);
         } else {
 #pragma unroll
-            for (int ix = 0; ix < M; ++ix) put(ix, b * hs[r * M + ix] + a.w1_f[ix] * (q + a.xi_f[ix] * jj));
+            for (int ix = 0; ix < M; ++ix) put(ix, a.b_f * hs[r * M + ix] + a.w1_f[ix] * (q + a.xi_f[ix] * jj));
         }
     }
 
     if (ACC) {
+        // fixed order: the lanes of each warp by a butterfly, then the warps (one FP64 operation
+        // of one lane costs the pipe as much as a warp's)
         const int T = W * NS * blockDim.z, t = threadIdx.x + W * (g + NS * threadIdx.z);
-        s_red[0][t] = valid ? (double)psd : 0.0;
-        s_red[1][t] = valid ? (double)psn : 0.0;
-        __syncthreads();
-        if (t < 32) {                                 // fixed order: strided sums, then the 32 of them
-            double d = 0.0, n = 0.0;
-            for (int k = t; k < T; k += 32) {
-                d += s_red[0][k];
-                n += s_red[1][k];
+        const int lanes = T - (t & ~31) < 32 ? T - (t & ~31) : 32;
+        const unsigned mask = lanes == 32 ? 0xffffffffu : (1u << lanes) - 1;
+        double d = valid ? (double)psd : 0.0, n = valid ? (double)psn : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double dd = __shfl_down_sync(mask, d, o), dnn = __shfl_down_sync(mask, n, o);
+            if (o < lanes) {
+                const bool in = (t & 31) + o < lanes;
+                d += in ? dd : 0.0;
+                n += in ? dnn : 0.0;
             }
-            s_red[0][t] = d;
-            s_red[1][t] = n;
+        }
+        if ((t & 31) == 0) {
+            s_red[0][t >> 5] = d;
+            s_red[1][t >> 5] = n;
         }
         __syncthreads();
         if (t == 0) {
-            double d = 0.0, n = 0.0;
-            for (int k = 0; k < 32 && k < T; ++k) {
+            for (int k = 1; 32 * k < T; ++k) {
                 d += s_red[0][k];
                 n += s_red[1][k];
             }
