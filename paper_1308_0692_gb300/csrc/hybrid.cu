@@ -118,11 +118,10 @@ __device__ __forceinline__ T warp_sum(T v)
 // ...; smaller ones: the source velocities split over 32 / lanes lane groups, the partial sums
 // combined by shuffles (every lane of the warp calls this).
 template <typename T>
-__device__ void project_warp(const HybTabT<T> &tb, int ti, const T *h, T *out)
+__device__ void project_warp(const HybTabT<T> &tb, const T *pt, int ti, const T *h, T *out)
 {
     const int lane = threadIdx.x & 31;
     const HybSetT<T> &Tg = tb.set[ti], &S = tb.set[ti ^ 1];
-    const T *pt = tb.pt[ti];
     const int nt = Tg.n, ns = S.n;
     if (ns > 16) {
         for (int b = lane; b < ns; b += 32) {
@@ -167,7 +166,7 @@ __device__ void neighbour_values(const HybArgs &a, int k, int sj, T *buf, T *tmp
         gather_cell(h, a.toff, k, tb.set[sj].n, buf);
     } else {
         gather_cell(h, a.toff, k, tb.set[sk].n, tmp);
-        project_warp(tb, sk, tmp, buf);
+        project_warp(tb, tb.pt[sk], sk, tmp, buf);
     }
 }
 
@@ -215,18 +214,44 @@ __device__ void face_moments(const HybSetT<T> &S, const T *v, int axis, bool pos
     m[2] = warp_sum(p2);
 }
 
+// This lane's part of sum nu_d (1, xi_x, xi_y) (p - n), p over the velocities of S moving along
+// +axis (values vp), n over those moving along -axis (values vn): the net exchange through
+// a face times dt / d.  Summed over the warp once for all the faces of a cell -- a warp sum is
+// five FP64 operations of all lanes, a third of an interface cell's when every flux had its own.
+template <typename T>
+__device__ __forceinline__ void face_exchange(const HybSetT<T> &S, const T *vp, const T *vn, int axis, T sign, T (&m)[3])
+{
+    for (int b = threadIdx.x & 31; b < S.n; b += 32) {
+        const int sd = axis == 0 ? S.sx[b] : S.sy[b];
+        if (sd == 0) continue;
+        const T nu = sign * (axis == 0 ? S.nux[b] : S.nuy[b]);
+        const T t = sd > 0 ? nu * vp[b] : -nu * vn[b];
+        m[0] += t;
+        m[1] += t * S.xi_x[b];
+        m[2] += t * S.xi_y[b];
+    }
+}
+
 template <typename T>
 struct HybShared {
-    T nbv[HWARPS][4][HMAXV];   // left, right, below, above: upwind values in the cell's set
-    T ph[HWARPS][HMAXV], nb[HWARPS][HMAXV];
-    T own[HWARPS][HMAXV], tmp[HWARPS][HMAXV];   // the cell's values; a neighbour's before projection
+    T nbv[HWARPS][2][HMAXV];   // the two cells of a face in one set
+    T own[HWARPS][HMAXV], tmp[HWARPS][HMAXV];   // values before projection
+};
+
+// Shared buffers of interface_cell: the cell's and its neighbours' values (left, right, below,
+// above), the neighbours' values in the cell's set, the cell's in the half-range one
+template <int N, typename T>
+struct IfShared {
+    static constexpr int NV = 4 * N * N, KV = (NV + 31) / 32;
+    static constexpr bool STAGED = N <= 4;               // the projection matrices fit beside them
+    T own[HWARPS][NV], raw[HWARPS][4][NV], seen[HWARPS][4][NV], ph[HWARPS][NV];
+    T pt[2][STAGED ? NV * N * N : 1];
 };
 
 // A cell with an interface face (a neighbour in the other set): one warp, warp `wi` of the
 // block's shared buffers; arithmetic in the storage type TS.
-template <typename TS>
-__device__ void interface_cell(const HybArgs &a, HybShared<TS> &sh, int wi, int c, double dt_dx, double dt_dy,
-                               int resid)
+template <int N, typename TS>
+__device__ void interface_cell(const HybArgs &a, IfShared<N, TS> &sh, int wi, int c, int resid)
 {
     using T = TS;
     const int lane = threadIdx.x & 31;
@@ -235,55 +260,79 @@ __device__ void interface_cell(const HybArgs &a, HybShared<TS> &sh, int wi, int 
     const int sj = a.half[c] ? 0 : 1;
     const HybSetT<T> &S = tb.set[sj];
     const HybSetT<T> &H = tb.set[0];
-    T *hc = sh.own[wi];
-    gather_cell(static_cast<const TS *>(a.h), a.toff, c, S.n, hc);
-    T *tmp = sh.tmp[wi];
+    constexpr int KV = IfShared<N, T>::KV;
+    const T *const pt[2] = {IfShared<N, T>::STAGED ? sh.pt[0] : tb.pt[0], IfShared<N, T>::STAGED ? sh.pt[1] : tb.pt[1]};
     const int x = c % nx, y = c / nx;
-    T(*nbv)[HMAXV] = sh.nbv[wi];
-    // upwind values: x (cavity only) and y neighbours in this cell's set, or the walls' ghosts;
     // the four faces as (axis, side, neighbour or -1)
-    int nbc[4] = {-1, -1, -1, -1};
-    if (a.cavity) {
-        if (x > 0) neighbour_values<TS>(a, nbc[0] = c - 1, sj, nbv[0], tmp);
-        else wall_ghost(a, S, hc, 2, nbv[0]);
-        if (x < nx - 1) neighbour_values<TS>(a, nbc[1] = c + 1, sj, nbv[1], tmp);
-        else wall_ghost(a, S, hc, 3, nbv[1]);
+    const int nbc[4] = {a.cavity && x > 0 ? c - 1 : -1, a.cavity && x < nx - 1 ? c + 1 : -1, y > 0 ? c - nx : -1,
+                        y < ny - 1 ? c + nx : -1};
+    // the values of the cell and its neighbours, each in its own set: every load issued before the
+    // first is used (gathered one after another, each a dependent chain of its own, they were most of the
+    // FP32 step's time on a small grid)
+    T *hc = sh.own[wi];
+    int set_of[4];
+    {
+        const TS *h = static_cast<const TS *>(a.h);
+        const TS *at[5];
+        int n[5];
+#pragma unroll
+        for (int f = 0; f < 5; ++f) {
+            const int k = f < 4 ? (nbc[f] >= 0 ? nbc[f] : c) : c, t = a.half[k] ? 0 : 1;
+            if (f < 4) set_of[f] = t;
+            at[f] = h + a.toff[k];
+            n[f] = f < 4 && nbc[f] < 0 ? 0 : tb.set[t].n;
+        }
+        T v[5][KV];
+#pragma unroll
+        for (int f = 0; f < 5; ++f)
+#pragma unroll
+            for (int i = 0; i < KV; ++i) v[f][i] = lane + 32 * i < n[f] ? (T)at[f][(long)HST * (lane + 32 * i)] : T(0);
+#pragma unroll
+        for (int f = 0; f < 5; ++f)
+#pragma unroll
+            for (int i = 0; i < KV; ++i)
+                if (lane + 32 * i < n[f]) (f < 4 ? sh.raw[wi][f] : hc)[lane + 32 * i] = v[f][i];
     }
-    if (y > 0) neighbour_values<TS>(a, nbc[2] = c - nx, sj, nbv[2], tmp);
-    else wall_ghost(a, S, hc, 0, nbv[2]);
-    if (y < ny - 1) neighbour_values<TS>(a, nbc[3] = c + nx, sj, nbv[3], tmp);
-    else wall_ghost(a, S, hc, 1, nbv[3]);
+    __syncwarp();
+    // upwind values: x (cavity only) and y neighbours in this cell's set, or the walls' ghosts
+    T *nbv[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        nbv[f] = sh.raw[wi][f];
+        if (nbc[f] < 0) {
+            if (f >= 2 || a.cavity) wall_ghost(a, S, hc, f < 2 ? f + 2 : f - 2, nbv[f]);
+        } else if (set_of[f] != sj) {
+            nbv[f] = sh.seen[wi][f];
+            project_warp(tb, pt[set_of[f]], set_of[f], sh.raw[wi][f], nbv[f]);
+        }
+    }
     // interface faces of a full-range cell: mass and momentum exchange made equal to the
     // half-range evaluation of the face
     T cr[3] = {0, 0, 0};
     bool any_if = false;
     if (sj == 1)
-        for (int f = 0; f < 4; ++f) any_if |= nbc[f] >= 0 && a.half[nbc[f]];
+        for (int f = 0; f < 4; ++f) any_if |= nbc[f] >= 0 && set_of[f] == 0;
     if (any_if) {
-        T *ph = sh.ph[wi], *nb = sh.nb[wi];
-        project_warp(tb, 1, hc, ph);                            // this cell seen in H
+        T *ph = sh.ph[wi];
+        project_warp(tb, pt[1], 1, hc, ph);                     // this cell seen in H
+#pragma unroll
         for (int f = 0; f < 4; ++f) {
-            if (nbc[f] < 0 || !a.half[nbc[f]]) continue;
+            if (nbc[f] < 0 || set_of[f] != 0) continue;
             const int axis = f >> 1;
             const bool lower = (f & 1) == 0;                  // the neighbour is on the lower side
-            neighbour_values<TS>(a, nbc[f], 0, nb, tmp);      // its own half-range values
-            T up[3], dn[3], got[3], sent[3];
-            face_moments(H, lower ? nb : ph, axis, true, up);
-            face_moments(H, lower ? ph : nb, axis, false, dn);
-            face_moments(S, nbv[f], axis, lower, got);
-            face_moments(S, hc, axis, !lower, sent);
-            const T fac = (T)(axis == 0 ? dt_dx : dt_dy);
-            for (int q = 0; q < 3; ++q) {
-                const T want = lower ? up[q] - dn[q] : dn[q] - up[q];
-                cr[q] += fac * (want - (got[q] - sent[q]));
-            }
+            const T *nb = sh.raw[wi][f];                      // its own half-range values
+            // the half-range evaluation of the face, less what this cell's set received and sent
+            face_exchange(H, lower ? nb : ph, lower ? ph : nb, axis, lower ? T(1) : T(-1), cr);
+            face_exchange(S, lower ? nbv[f] : hc, lower ? hc : nbv[f], axis, lower ? T(-1) : T(1), cr);
         }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) cr[q] = warp_sum(cr[q]);
     }
     // transport, moments, relaxation
-    T hs[(HMAXV + 31) / 32];
+    T hs[KV];
     T rho = 0, jx = 0, jy = 0;
 #pragma unroll
-    for (int i = 0; i < (HMAXV + 31) / 32; ++i) {
+    for (int i = 0; i < KV; ++i) {
         const int b = lane + 32 * i;
         T v = 0;
         if (b < S.n) {
@@ -314,7 +363,7 @@ __device__ void interface_cell(const HybArgs &a, HybShared<TS> &sh, int wi, int 
     const T om = (T)a.omega;
     T pd = 0, pn = 0;
 #pragma unroll
-    for (int i = 0; i < (HMAXV + 31) / 32; ++i) {
+    for (int i = 0; i < KV; ++i) {
         const int b = lane + 32 * i;
         if (b < S.n) {
             const T heq = S.w[b] * (rho + S.xi_x[b] * jx + S.xi_y[b] * jy);
@@ -358,8 +407,12 @@ struct PlainArgs {
     int nx, ny, cavity, homogeneous;
     TC omega, b, u_bottom, u_top, inv_u_ref;   // b = 1 - omega
     double inv_dx_wall, inv_dy_wall;   // 1 / sum_{xi > 0} xi w over the set, per axis
-    TC xi[12], w1[12], nux[12], nuy[12];
-    TC a0[144];                        // 1 - nu_x - nu_y per velocity a = iy M + ix
+    TC xi[12], w1[12], wxi[12], omw[12];   // omw: (omega / s) w1, wxi: w1 xi
+    // transport coefficients, scaled by s: 1, or in FP64 1 - omega unless that is small (fold; then
+    // the relaxation only adds to the scaled transported values)
+    TC nux[12], nuy[12];
+    TC a0[144];                        // s (1 - nu_x - nu_y) per velocity a = iy M + ix
+    int fold;
 };
 
 // blocks of four warps: G warps per tile, 4 / G tiles per block
@@ -401,23 +454,29 @@ __device__ __forceinline__ void plain_tiles(const PlainArgs<TC> &p, const int2 *
     if (__syncthreads_or((int)(on && (wl || wr || wb || wt)))) {
         double pw[4] = {0.0, 0.0, 0.0, 0.0};     // outflow through the bottom, top, left, right walls
         // products and the sums over one velocity row in the arithmetic type, the sums over
-        // rows and warps in FP64 (as the single-domain kernels do; per-velocity FP64 sums kept
-        // the FP64 pipe of the FP32 hybrid step 38 % busy)
+        // rows and warps in FP64 (as the single-domain kernels do), of the lanes at each wall
+        auto sum_rows = [&](int lo, int hi, double &out) {     // over ix in [lo, hi): |xi_x| h
 #pragma unroll
-        for (int r = 0; r < RPL; ++r) {
-            const int iy = g * RPL + r;
-            TC ys = 0, ls = 0, rs = 0;
+            for (int r = 0; r < RPL; ++r) {
+                TC t = 0;
 #pragma unroll
-            for (int ix = 0; ix < M; ++ix) {
-                const TC v = h[oc + (long)HST * (iy * M + ix)];
-                ys += v;
-                if (ix < HALF) ls -= p.xi[ix] * v;
-                if (ix >= M - HALF) rs += p.xi[ix] * v;
+                for (int ix = 0; ix < M; ++ix)
+                    if (ix >= lo && ix < hi) t += (ix < HALF ? -p.xi[ix] : p.xi[ix]) * h[oc + (long)HST * ((g * RPL + r) * M + ix)];
+                out += (double)t;
             }
-            if (iy < HALF) pw[0] -= (double)(p.xi[iy] * ys);
-            if (iy >= M - HALF) pw[1] += (double)(p.xi[iy] * ys);
-            pw[2] += (double)ls;
-            pw[3] += (double)rs;
+        };
+        if (wl) sum_rows(0, HALF, pw[2]);
+        if (wr) sum_rows(M - HALF, M, pw[3]);
+        if (wb || wt) {
+#pragma unroll
+            for (int r = 0; r < RPL; ++r) {
+                const int iy = g * RPL + r;
+                TC t = 0;
+#pragma unroll
+                for (int ix = 0; ix < M; ++ix) t += h[oc + (long)HST * (iy * M + ix)];
+                if (iy < HALF) pw[0] -= (double)(p.xi[iy] * t);
+                if (iy >= M - HALF) pw[1] += (double)(p.xi[iy] * t);
+            }
         }
         if (G > 1) {
 #pragma unroll
@@ -439,8 +498,9 @@ __device__ __forceinline__ void plain_tiles(const PlainArgs<TC> &p, const int2 *
 
     // ---- transport and moment sums ----
     // h* = (1 - nu_x - nu_y) h + nu_x h_x + nu_y h_y; rho, j_x per velocity, j_y per row.
-    // The wall ghosts are formed only in tiles that touch a wall (WALLS): as a select in every
-    // tile they doubled the FP64 operations of the step.
+    // The wall ghosts are formed only in tiles that touch a wall of that axis (XW, YW): as a
+    // select in every tile they doubled the FP64 operations of the step.  FP64 takes seven operations
+    // per velocity and a few per row, as step_tile.cuh.
     // the FP32 march's correction sweeps drop the walls' driving terms and add the defect; the
     // FP64 march never does (its kernels carry no code for it)
     constexpr bool MIXED = std::is_same<TC, float>::value;
@@ -448,12 +508,19 @@ __device__ __forceinline__ void plain_tiles(const PlainArgs<TC> &p, const int2 *
     const TC drive = (MIXED && p.homogeneous) ? TC(0) : p.inv_u_ref;     // the walls' driving term
     TC hs[RPL * M];
     TC R = 0, X = 0, Y = 0;
-    auto transport = [&](auto walls_tag) {
-        constexpr bool WALLS = decltype(walls_tag)::value;
+    auto transport = [&](auto xwalls_tag, auto ywalls_tag) {
+        constexpr bool XW = decltype(xwalls_tag)::value, YW = decltype(ywalls_tag)::value;
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
             const int iy = g * RPL + r;
             const TC nuy = p.nuy[iy], wy = p.w1[iy];
+            const bool ywall = YW && (iy >= M - HALF ? wb : iy < HALF && wt);
+            TC gy0 = 0, gy1 = 0;                      // ghost w_x (gy0 + xi_x gy1) of a y wall
+            if (YW) {
+                const TC d = iy < HALF ? rw[1] : rw[0], u = iy < HALF ? ut : ub;
+                gy0 = wy * d;
+                gy1 = wy * (d * u + u * drive);
+            }
             TC Rr = 0, Xr = 0;
 #pragma unroll
             for (int ix = 0; ix < M; ++ix) {
@@ -464,47 +531,63 @@ __device__ __forceinline__ void plain_tiles(const PlainArgs<TC> &p, const int2 *
                     TC hx = h0;
                     if (ix >= M - HALF) {
                         hx = h[ol + a];
-                        if (WALLS && wl) hx = p.w1[ix] * wy * rw[2];          // side walls at rest
+                        if (XW && wl) hx = p.w1[ix] * (wy * rw[2]);           // side walls at rest
                     } else if (ix < HALF) {
                         hx = h[orr + a];
-                        if (WALLS && wr) hx = p.w1[ix] * wy * rw[3];
+                        if (XW && wr) hx = p.w1[ix] * (wy * rw[3]);
                     }
                     v = fma_(p.nux[ix], hx, v);
                 }
                 TC hy = h0;
-                if (iy >= M - HALF) {
-                    hy = h[od + a];
-                    if (WALLS && wb) hy = p.w1[ix] * wy * (rw[0] * (TC(1) + p.xi[ix] * ub) + p.xi[ix] * ub * drive);
-                } else if (iy < HALF) {
-                    hy = h[ou + a];
-                    if (WALLS && wt) hy = p.w1[ix] * wy * (rw[1] * (TC(1) + p.xi[ix] * ut) + p.xi[ix] * ut * drive);
-                }
+                if (iy >= M - HALF) hy = h[od + a];
+                else if (iy < HALF) hy = h[ou + a];
+                if (YW && ywall) hy = fma_(p.wxi[ix], gy1, p.w1[ix] * gy0);
                 v = fma_(nuy, hy, v);
                 hs[r * M + ix] = v;
                 Rr += v;
-                Xr = fma_(p.xi[ix], v, Xr);
+                if (MIXED) Xr = fma_(p.xi[ix], v, Xr);
+                else X = fma_(p.xi[ix], v, X);
             }
             R += Rr;
-            X += Xr;
+            if (MIXED) X += Xr;
             Y = fma_(p.xi[iy], Rr, Y);
         }
     };
-    if (__any_sync(0xffffffffu, wl || wr || wb || wt)) transport(std::true_type{});
-    else transport(std::false_type{});
+    // (warp-uniform: a warp's tile touches no wall, side walls only, or the bottom or top; FP32, where
+    // the ghosts cost little, keeps one form for all walls and its registers)
+    if (__any_sync(0xffffffffu, wb || wt || (MIXED && (wl || wr)))) transport(std::true_type{}, std::true_type{});
+    else if (!MIXED && __any_sync(0xffffffffu, wl || wr)) transport(std::true_type{}, std::false_type{});
+    else transport(std::false_type{}, std::false_type{});
     if (G > 1) {
         s_x[tl][g][0][lane] = R;
         s_x[tl][g][1][lane] = X;
         s_x[tl][g][2][lane] = Y;
         __syncthreads();
-        R = X = Y = 0;
+        if (!MIXED && G == 4) {            // FP64: warp k < 3 sums moment k for all four
+            if (g < 3) {
+                double t = 0.0;
 #pragma unroll
-        for (int q = 0; q < G; ++q) {
-            R += (TC)s_x[tl][q][0][lane];
-            X += (TC)s_x[tl][q][1][lane];
-            Y += (TC)s_x[tl][q][2][lane];
+                for (int q = 0; q < G; ++q) t += s_x[tl][q][g][lane];
+                s_x[tl][g][3][lane] = t;
+            }
+            __syncthreads();
+            R = (TC)s_x[tl][0][3][lane];
+            X = (TC)s_x[tl][1][3][lane];
+            Y = (TC)s_x[tl][2][3][lane];
+        } else {
+            R = X = Y = 0;
+#pragma unroll
+            for (int q = 0; q < G; ++q) {
+                R += (TC)s_x[tl][q][0][lane];
+                X += (TC)s_x[tl][q][1][lane];
+                Y += (TC)s_x[tl][q][2][lane];
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
+    if (!MIXED && !p.fold)
+#pragma unroll
+        for (int k = 0; k < RPL * M; ++k) hs[k] *= p.b;
 
     // ---- relaxation h' = (1 - omega) h* + omega w (rho + xi . j), store, residual sums ----
     TC pd = 0, pn = 0;
@@ -512,12 +595,18 @@ __device__ __forceinline__ void plain_tiles(const PlainArgs<TC> &p, const int2 *
 #pragma unroll
     for (int r = 0; r < RPL; ++r) {
         const int iy = g * RPL + r;
-        const TC ow = p.omega * p.w1[iy];
+        const TC ow = MIXED ? p.omega * p.w1[iy] : p.omw[iy];
         const TC A = ow * fma_(p.xi[iy], Y, R), B = ow * X;
 #pragma unroll
         for (int ix = 0; ix < M; ++ix) {
             const long a = (long)HST * (iy * M + ix);
-            TC o = fma_(p.b, hs[r * M + ix], p.w1[ix] * fma_(p.xi[ix], B, A));
+            TC o;
+            if (MIXED) {
+                o = fma_(p.b, hs[r * M + ix], p.w1[ix] * fma_(p.xi[ix], B, A));
+            } else {
+                o = fma_(p.w1[ix], A, hs[r * M + ix]);
+                if (2 * ix + 1 != M) o = fma_(p.wxi[ix], B, o);
+            }
             if (MIXED && src) o += (TC)src[a];
             if (on) p.hn[oc + a] = o;
             if (resid) {
@@ -563,27 +652,39 @@ struct StepLists {
 };
 
 // blocks a SM the FP32 build asks for: eight (64 registers a thread) where that does not
-// spill, six for the 100-velocity half-range set; FP64 as the compiler chooses
+// spill, six for the 100- and 144-velocity half-range sets; FP64 as the compiler chooses
 template <int N, typename TS>
-constexpr int hybrid_min_blocks() { return sizeof(TS) == 8 ? 1 : (N == 5 ? 6 : 8); }
+constexpr int hybrid_min_blocks() { return sizeof(TS) == 8 ? 1 : (N >= 5 ? 6 : 8); }
 
 template <int N, typename TS>
 __global__ void __launch_bounds__(32 * HWARPS, hybrid_min_blocks<N, TS>()) hybrid_step_kernel(const HybArgs a, const PlainArgs<TS> ph,
                                                                    const PlainArgs<TS> pf, const StepLists L,
-                                                                   double dt_dx, double dt_dy, int resid)
+                                                                   int resid)
 {
     constexpr int GH = half_warps(N);
     __shared__ union {
-        HybShared<TS> sh;
+        IfShared<N, TS> sh;
         double hx[HWARPS / GH][GH][4][32];
         double fx[HWARPS][1][4][32];
     } u;
     const int bid = (int)blockIdx.x;
     const int ifb = (L.ncells + HWARPS - 1) / HWARPS;
     const int hbk = (L.ntiles[0] + HWARPS / GH - 1) / (HWARPS / GH);
+    // the next step's blocks are set up while this one runs (for the interface cells with the
+    // projection matrices in shared memory) and wait for it before they read the state
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (IfShared<N, TS>::STAGED && bid < ifb) {
+        const HybTabT<TS> &tb = *static_cast<const HybTabT<TS> *>(a.tab);
+        for (int k = threadIdx.x; k < 4 * N * N * N * N; k += 32 * HWARPS) {
+            u.sh.pt[0][k] = tb.pt[0][k];
+            u.sh.pt[1][k] = tb.pt[1][k];
+        }
+        __syncthreads();
+    }
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     if (bid < ifb) {
         const int wi = threadIdx.x >> 5, ci = bid * HWARPS + wi;
-        if (ci < L.ncells) interface_cell<TS>(a, u.sh, wi, L.cells[ci], dt_dx, dt_dy, resid);    // whole warps
+        if (ci < L.ncells) interface_cell<N, TS>(a, u.sh, wi, L.cells[ci], resid);    // whole warps
     } else if (bid < ifb + hbk) {
         plain_tiles<2 * N, GH>(ph, L.tiles[0], L.ntiles[0], bid - ifb, resid, u.hx);
     } else {
@@ -593,26 +694,34 @@ __global__ void __launch_bounds__(32 * HWARPS, hybrid_min_blocks<N, TS>()) hybri
 
 template <int N, typename TS>
 cudaError_t launch_step_n(const HybArgs &a, const PlainArgs<TS> &ph, const PlainArgs<TS> &pf, const StepLists &L,
-                          double dt_dx, double dt_dy, int resid, cudaStream_t st)
+                          int resid, cudaStream_t st)
 {
     constexpr int GH = half_warps(N);
     const int blocks = (L.ncells + HWARPS - 1) / HWARPS + (L.ntiles[0] + HWARPS / GH - 1) / (HWARPS / GH) +
                        (L.ntiles[1] + HWARPS - 1) / HWARPS;
     if (blocks == 0) return cudaSuccess;
-    hybrid_step_kernel<N, TS><<<blocks, 32 * HWARPS, 0, st>>>(a, ph, pf, L, dt_dx, dt_dy, resid);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(32 * HWARPS);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = st != nullptr ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, hybrid_step_kernel<N, TS>, a, ph, pf, L, resid);
 }
 
 template <typename TS>
 cudaError_t launch_hybrid_step(int n, const HybArgs &a, const PlainArgs<TS> &ph, const PlainArgs<TS> &pf,
-                               const StepLists &L, double dt_dx, double dt_dy, int resid, cudaStream_t st)
+                               const StepLists &L, int resid, cudaStream_t st)
 {
     switch (n) {
-    case 2: return launch_step_n<2, TS>(a, ph, pf, L, dt_dx, dt_dy, resid, st);
-    case 3: return launch_step_n<3, TS>(a, ph, pf, L, dt_dx, dt_dy, resid, st);
-    case 4: return launch_step_n<4, TS>(a, ph, pf, L, dt_dx, dt_dy, resid, st);
-    case 5: return launch_step_n<5, TS>(a, ph, pf, L, dt_dx, dt_dy, resid, st);
-    case 6: return launch_step_n<6, TS>(a, ph, pf, L, dt_dx, dt_dy, resid, st);
+    case 2: return launch_step_n<2, TS>(a, ph, pf, L, resid, st);
+    case 3: return launch_step_n<3, TS>(a, ph, pf, L, resid, st);
+    case 4: return launch_step_n<4, TS>(a, ph, pf, L, resid, st);
+    case 5: return launch_step_n<5, TS>(a, ph, pf, L, resid, st);
+    case 6: return launch_step_n<6, TS>(a, ph, pf, L, resid, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -766,30 +875,30 @@ __global__ void __launch_bounds__(32 * HWARPS) hybrid_face_flux_kernel(const Hyb
     if (lane == 0) pxy[k] = u_ref * (up + dn);
 }
 
-// (u_x, u_y) of every cell from its own set: u = u_ref sum xi h / (1 + u_ref sum h)
-__global__ void __launch_bounds__(32 * HWARPS) hybrid_velocity_kernel(const HybArgs a, double u_ref, double *ux,
-                                                                       double *uy)
+// (u_x, u_y) of every cell from its own set: u = u_ref sum xi h / (1 + u_ref sum h); one thread
+// a cell (consecutive cells of a tile are consecutive in memory)
+__global__ void __launch_bounds__(128) hybrid_velocity_kernel(const HybArgs a, int m_half, double u_ref, double *ux, double *uy)
 {
-    const int lane = threadIdx.x & 31;
-    const int c = blockIdx.x * HWARPS + (threadIdx.x >> 5);
+    const int c = blockIdx.x * 128 + threadIdx.x;
     if (c >= a.nx * a.ny) return;
-    const HybSetT<double> &S = static_cast<const HybTabT<double> *>(a.tab)->set[a.half[c] ? 0 : 1];
+    const int t = a.half[c] ? 0 : 1, m = t == 0 ? m_half : m_half / 2;
+    const HybSetT<double> &S = static_cast<const HybTabT<double> *>(a.tab)->set[t];
     const double *hc = static_cast<const double *>(a.h) + a.toff[c];
     double s0 = 0.0, sx = 0.0, sy = 0.0;
-    for (int b = lane; b < S.n; b += 32) {
-        const double v = hc[(long)HST * b];
-        s0 += v;
-        sx += S.xi_x[b] * v;
-        sy += S.xi_y[b] * v;
+    for (int iy = 0; iy < m; ++iy) {
+        double row = 0.0;
+#pragma unroll 4
+        for (int ix = 0; ix < m; ++ix) {
+            const double v = hc[(long)HST * (iy * m + ix)];
+            row += v;
+            sx += S.xi_x[ix] * v;
+        }
+        s0 += row;
+        sy += S.xi_y[iy * m] * row;
     }
-    s0 = warp_sum(s0);
-    sx = warp_sum(sx);
-    sy = warp_sum(sy);
-    if (lane == 0) {
-        const double rho = 1.0 + u_ref * s0;
-        ux[c] = u_ref * sx / rho;
-        uy[c] = u_ref * sy / rho;
-    }
+    const double rho = 1.0 + u_ref * s0;
+    ux[c] = u_ref * sx / rho;
+    uy[c] = u_ref * sy / rho;
 }
 
 }  // namespace
@@ -917,16 +1026,20 @@ PlainArgs<TC> plain_args(const lbm_hybrid *hb, int set, const HybArgs &a)
     p.inv_dy_wall = hb->inv_dy_wall[set];
     const int m = hb->m1[set];
     double nux[12], nuy[12];
+    p.fold = sizeof(TC) == 8 && 1.0 - hb->omega >= 0.0625;
+    const double s = p.fold ? 1.0 - hb->omega : 1.0;
     for (int i = 0; i < m; ++i) {
         nux[i] = p.cavity ? std::fabs(hb->x1[set][i]) * hb->dt / hb->dx : 0.0;
         nuy[i] = std::fabs(hb->x1[set][i]) * hb->dt / hb->dy;
         p.xi[i] = (TC)hb->x1[set][i];
         p.w1[i] = (TC)hb->w1[set][i];
-        p.nux[i] = (TC)nux[i];
-        p.nuy[i] = (TC)nuy[i];
+        p.wxi[i] = (TC)(hb->w1[set][i] * hb->x1[set][i]);
+        p.omw[i] = (TC)(hb->omega / s * hb->w1[set][i]);
+        p.nux[i] = (TC)(s * nux[i]);
+        p.nuy[i] = (TC)(s * nuy[i]);
     }
     for (int iy = 0; iy < m; ++iy)
-        for (int ix = 0; ix < m; ++ix) p.a0[iy * m + ix] = (TC)(1.0 - nux[ix] - nuy[iy]);
+        for (int ix = 0; ix < m; ++ix) p.a0[iy * m + ix] = (TC)(s * (1.0 - nux[ix] - nuy[iy]));
     return p;
 }
 
@@ -943,10 +1056,8 @@ cudaError_t hybrid_launch(const lbm_hybrid *hb, const HybArgs &a0, int resid)
         L.tiles[t] = hb->d_tiles[t];
         L.ntiles[t] = hb->n_tiles[t];
     }
-    // the interface faces' dt / dx and dt / dy, divided once here (the device's FP64 divide
-    // would run on every lane of every interface warp)
-    return launch_hybrid_step<TS>(hb->n_half, a, plain_args<TS>(hb, 0, a), plain_args<TS>(hb, 1, a), L,
-                                  hb->dt / hb->dx, hb->dt / hb->dy, resid, hb->stream);
+    return launch_hybrid_step<TS>(hb->n_half, a, plain_args<TS>(hb, 0, a), plain_args<TS>(hb, 1, a), L, resid,
+                                  hb->stream);
 }
 
 // the two-stage reduction of the residual partials into d_res[0..1]
@@ -1469,19 +1580,16 @@ lbm_status lbm_hybrid_velocity(lbm_hybrid *hb, double *ux, double *uy)
 {
     if (!hb || !ux || !uy) return hfail(LBM_EINVAL, "NULL argument");
     const int nc = hb->nx * hb->ny;
-    double *d = nullptr;
+    double *d = hb->d_part;               // the residual partials, reduced by the end of every step call
     const double *h64 = nullptr;
     cudaError_t e = hybrid_state_f64(hb, &h64);
-    if (e == cudaSuccess) e = cudaMalloc(&d, sizeof(double) * 2 * nc);
     if (e == cudaSuccess) {
-        hybrid_velocity_kernel<<<(nc + HWARPS - 1) / HWARPS, 32 * HWARPS, 0, hb->stream>>>(hargs(hb, h64), hb->u_ref, d,
-                                                                                            d + nc);
+        hybrid_velocity_kernel<<<(nc + 127) / 128, 128, 0, hb->stream>>>(hargs(hb, h64), hb->m1[0], hb->u_ref, d, d + nc);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(ux, d, sizeof(double) * nc, cudaMemcpyDeviceToHost, hb->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(uy, d + nc, sizeof(double) * nc, cudaMemcpyDeviceToHost, hb->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(hb->stream);
-    if (d) cudaFree(d);
     return e == cudaSuccess ? LBM_OK : hfail(LBM_ECUDA, std::string("hybrid velocity: ") + cudaGetErrorString(e));
 }
 
