@@ -23,6 +23,9 @@ cudaError_t launch_step_f32_small(int m, int ns, bool resid, const StepArgs &a, 
 cudaError_t launch_step_f32_large(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s);
 cudaError_t launch_defect_f32(int m, int ns, const StepArgs &a, cudaStream_t s);
 cudaError_t launch_correct_f32(int m, int ns, bool resid, const StepArgs &a, cudaStream_t s);
+bool prepare_column(bool dp, int m, int ny);
+int column_blocks();
+cudaError_t launch_column(bool dp, int m, const StepArgs &a, int steps, int resid, cudaStream_t s);
 cudaError_t launch_step_f32_tma(int m, int g, bool resid, const StepArgs &a, int grid, cudaStream_t s,
                                bool merged);
 cudaError_t prepare_step_f32_tma(int m, int g);
@@ -58,6 +61,7 @@ struct lbm_sim {
     int lanes;            // warps per 32-cell segment of the step kernel (load paths 0, 1: velocity slices)
     bool lanes_set;       // lanes chosen by lbm_set_variant; else tile_plan picks the slices of load path 0
     int slices;           // velocity slices of load paths 0 and 1
+    bool column;          // a one-column channel whose steps run together on a cluster (step_column.cu)
     int prefetch;         // load path of the wall-free cells (lbm_set_variant)
     int splitting;        // LBM_SPLIT_LIE (stored state h) or LBM_SPLIT_STRANG[_EXACT] (stored g = R(dt/2) h)
     int order;            // transport order: 1 (first-order upwind, the paper's) or 2
@@ -433,6 +437,13 @@ TilePlan tile_plan(bool dp, int m, long ncells)
     return {6, 16, 1};
 }
 
+// Longest one-column channel whose steps run together on a cluster (step_column.cu): beyond, the
+// cluster's 16 SMs take longer than the launches of step_tile.cuh over all of them.  Measured, us
+// per step, cluster / tiles: FP64 M = 8 at 100, 320, 500 cells 2.9 / 6.7, 4.7 / 6.5, 6.9 / 6.3;
+// M = 12 at 200, 320 6.1 / 8.5, 8.5 / 8.5; M = 4 at 500 2.7 / 4.4; FP32 M = 8 at 100, 500 1.5 / 2.7,
+// 2.7 / 2.6; M = 12 at 320, 500 2.9 / 3.8, 3.9 / 3.8.
+int column_cells(bool dp, int m) { return m == 12 ? (dp ? 300 : 450) : m == 8 ? 450 : 512; }
+
 // the same for slices the caller chose (lbm_set_variant)
 TilePlan tile_plan_for(bool dp, int ns) { return dp ? TilePlan{ns, 8, ns == 1 ? 4 : 1} : TilePlan{ns, ns >= 6 ? 16 : 32, ns == 1 ? 2 : 1}; }
 
@@ -456,7 +467,19 @@ void drop_graphs_fwd(lbm_sim *s) { drop_graphs(s); }
 cudaError_t enqueue_steps(lbm_sim *s, long first, long count, int cur, cudaStream_t st)
 {
     StepArgs a = s->args;
-    for (long i = 0; i < count; ++i) {
+    const long K = s->prob.residual_every;
+    for (long i = 0; s->column && i < count;) {       // the steps up to the next residual in one launch
+        const long n = std::min({count - i, K - (first + i - 1) % K, 1L << 20});
+        const bool resid = (first + i + n - 1) % K == 0;
+        a.h = s->buf[cur];
+        a.hn = s->buf[cur ^ (int)(n & 1)];
+        cudaError_t e = launch_column(s->prob.prec == LBM_FP64, s->vs.m, a, (int)n, resid, st);
+        if (e == cudaSuccess && resid) e = launch_finalize_residual(s->partials, s->nparts_step, s->result, st);
+        if (e != cudaSuccess) return e;
+        cur ^= (int)(n & 1);
+        i += n;
+    }
+    for (long i = 0; !s->column && i < count; ++i) {
         const long idx = first + i;
         const bool resid = idx % s->prob.residual_every == 0;
         a.h = s->buf[cur];
@@ -569,6 +592,9 @@ lbm_status set_lanes(lbm_sim *s, int lanes)
         s->args.tile_r = t.r;
         s->nparts_step = s->grid = (int)tile_blocks(nx, ny, t.w, t.r);
     }
+    s->column = s->order == 1 && s->prefetch == 0 && !s->lanes_set && !cav && nx == 1 && ny <= column_cells(s->prob.prec == LBM_FP64, s->vs.m) &&
+                prepare_column(s->prob.prec == LBM_FP64, s->vs.m, ny);
+    if (s->column) s->nparts_step = column_blocks();
     if (s->nparts_step > s->npartials) return fail(LBM_EINVAL, "internal: residual partials overflow");
     return LBM_OK;
 }
@@ -746,6 +772,7 @@ lbm_status lbm_init(const lbm_vset *vs, const lbm_problem *prob, const double *i
     s->stream = (cudaStream_t)stream;
     s->lanes = default_lanes_per_cell(prob->prec, vs->m);
     s->lanes_set = false;
+    s->column = false;
     s->prefetch = 0;
     s->splitting = LBM_SPLIT_LIE;
     s->order = 1;
@@ -849,7 +876,7 @@ lbm_status lbm_step(lbm_sim *s, long nsteps)
     // whole residual intervals replay a captured graph (not on the legacy stream, and not
     // while the caller is capturing this stream: then the launches go into their graph)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    bool graphs = s->stream != nullptr && K >= 2;
+    bool graphs = s->stream != nullptr && K >= 2 && !s->column;
     if (graphs && cudaStreamIsCapturing(s->stream, &cap) != cudaSuccess) graphs = false;
     if (cap != cudaStreamCaptureStatusNone) graphs = false;
     long i = 0;
@@ -872,13 +899,13 @@ lbm_status lbm_step(lbm_sim *s, long nsteps)
             i += K;
             continue;
         }
-        const long idx = s->step + 1;
-        cudaError_t e = enqueue_steps(s, idx, 1, s->cur, s->stream);
+        const long n = s->column ? std::min({nsteps - i, K - s->step % K, 1L << 20}) : 1;   // one launch
+        cudaError_t e = enqueue_steps(s, s->step + 1, n, s->cur, s->stream);
         if (e != cudaSuccess) return cuda_fail(e, "launching the step kernels");
-        if (idx % K == 0) s->resid_step = idx;
-        s->cur ^= 1;
-        s->step = idx;
-        ++i;
+        s->cur ^= (int)(n & 1);
+        s->step += n;
+        if (s->step % K == 0) s->resid_step = s->step;
+        i += n;
     }
     return LBM_OK;
 }
