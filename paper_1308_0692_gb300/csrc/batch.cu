@@ -2408,11 +2408,15 @@ lbm_status lbm_batch_warm_start(lbm_batch *b, int i, lbm_mlp *mlp, double kn, do
     const BatchInst &I = b->inst[i];
     if (!I.cavity) return bfail(LBM_EINVAL, "the warm-start network is trained on cavities");
     float *feat = b->d_scratch, *pred = b->d_scratch + 4 * I.ncells;
+    // the network runs on its own stream, between what the batch's stream holds now and the
+    // reconstruction
+    cudaError_t e = stream_after(mlp_stream(mlp), b->stream);
+    if (e != cudaSuccess) return bfail(LBM_ECUDA, std::string("warm start of an instance: ") + cudaGetErrorString(e));
     lbm_status st = lbm_mlp_features(mlp, I.nx, I.ny, kn, u_w, feat);
     if (st == LBM_OK) st = lbm_mlp_forward(mlp, feat, (int)I.ncells, pred);
+    e = stream_after(b->stream, mlp_stream(mlp));
+    if (e != cudaSuccess) cudaStreamSynchronize(mlp_stream(mlp));    // nothing outlives the call
     if (st != LBM_OK) return st;
-    // the MLP runs on its own stream: order the reconstruction after it
-    cudaError_t e = cudaDeviceSynchronize();
     if (e == cudaSuccess)
         e = launch_warm_state(pred, I.nx, I.ny, I.ncells, I.nx, b->m, b->d_tab, b->d_tab + LBM_MAX_M,
                               u_w * I.inv_u_ref, (float *)b->buf[0] + I.off, LBM_FP32_PERTURB, b->stream,

@@ -91,6 +91,8 @@ struct lbm_sim {
     StepArgs args;        // launch arguments except the buffer pointers
     cudaGraphExec_t graph[2];  // residual_every steps starting from buffer 0 / 1
     bool graph_ok[2];
+    cudaGraphExec_t cgraph[2][2];  // residual_every correction steps: state buffer, starting correction buffer
+    bool cgraph_ok[2][2];
     cudaStream_t cap_stream;   // private stream the graphs are captured on (created on first use)
     long step;
     long resid_step;
@@ -458,6 +460,10 @@ void drop_graphs(lbm_sim *s)
     for (int p = 0; p < 2; ++p) {
         if (s->graph_ok[p]) cudaGraphExecDestroy(s->graph[p]);
         s->graph_ok[p] = false;
+        for (int q = 0; q < 2; ++q) {
+            if (s->cgraph_ok[p][q]) cudaGraphExecDestroy(s->cgraph[p][q]);
+            s->cgraph_ok[p][q] = false;
+        }
     }
 }
 
@@ -784,6 +790,7 @@ lbm_status lbm_init(const lbm_vset *vs, const lbm_problem *prob, const double *i
     s->cur = 0;
     s->host_res = nullptr;
     s->graph_ok[0] = s->graph_ok[1] = false;
+    for (auto &g : s->cgraph_ok) g[0] = g[1] = false;
     s->cap_stream = nullptr;
     s->owns = device_buf == nullptr;
     s->bytes = L.total;
@@ -1034,15 +1041,17 @@ lbm_status lbm_solve(lbm_sim *s, double tol, long max_steps, int refine_sweeps, 
                 }
                 return cudaSuccess;
             };
-            // the intervals replay CUDA graphs (captured on the private stream, one per
-            // starting buffer); direct launches if a capture fails
-            cudaGraphExec_t cg[2] = {nullptr, nullptr};
+            // the intervals replay CUDA graphs (captured on the private stream, one per state buffer and
+            // starting correction buffer, kept with the sim: capturing one for every sweep took longer
+            // than its interval on a small grid); direct launches if a capture fails
+            auto &cg = s->cgraph[s->cur];
+            auto &cg_ok = s->cgraph_ok[s->cur];
             bool use_graphs = K >= 2 && make_capture_stream(s) == cudaSuccess;
             long k = 0;
             double cbest = INFINITY;
             int cflat = 0;
             while (k < max_steps) {
-                if (use_graphs && !cg[cc]) {
+                if (use_graphs && !cg_ok[cc]) {
                     cudaGraph_t gr = nullptr;
                     cudaError_t ec = cudaStreamBeginCapture(s->cap_stream, cudaStreamCaptureModeThreadLocal);
                     if (ec == cudaSuccess) {
@@ -1052,27 +1061,19 @@ lbm_status lbm_solve(lbm_sim *s, double tol, long max_steps, int refine_sweeps, 
                     }
                     if (ec == cudaSuccess) ec = cudaGraphInstantiate(&cg[cc], gr, 0);
                     if (gr) cudaGraphDestroy(gr);
+                    cg_ok[cc] = ec == cudaSuccess;
                     if (ec != cudaSuccess) {
                         cudaGetLastError();
-                        cg[cc] = nullptr;
                         use_graphs = false;
                     }
                 }
                 e = use_graphs ? cudaGraphLaunch(cg[cc], s->stream) : enqueue_interval(cc, s->stream);
-                if (e != cudaSuccess) {
-                    for (auto &x : cg)
-                        if (x) cudaGraphExecDestroy(x);
-                    return cuda_fail(e, "launching the correction march");
-                }
+                if (e != cudaSuccess) return cuda_fail(e, "launching the correction march");
                 cc ^= (int)(K & 1);
                 k += K;
                 double rr[4];
                 st = read_result(s, rr);
-                if (st != LBM_OK) {
-                    for (auto &x : cg)
-                        if (x) cudaGraphExecDestroy(x);
-                    return st;
-                }
+                if (st != LBM_OK) return st;
                 // change per step relative to ||h||, 10x below tol: the correction's own error
                 // is its per-step change times the conditioning of the slow modes (~1e3)
                 const double change = std::sqrt(rr[0]) / hnorm;
@@ -1084,8 +1085,6 @@ lbm_status lbm_solve(lbm_sim *s, double tol, long max_steps, int refine_sweeps, 
                     break;
                 }
             }
-            for (auto &x : cg)
-                if (x) cudaGraphExecDestroy(x);
             out.correction_steps += k;
             e = launch_add_f32((float *)H, (const float *)C[cc], (long)s->nv * s->ncells, s->stream);
             if (e != cudaSuccess) return cuda_fail(e, "applying the correction");
@@ -1113,13 +1112,15 @@ lbm_status lbm_warm_start(lbm_sim *s, lbm_mlp *mlp, double kn, double u_w)
     if (s->prob.geom != LBM_CAVITY) return fail(LBM_EINVAL, "the warm-start network is trained on cavities");
     float *feat = (float *)s->moments;                  // scratch: 16 B + 24 B per cell <= 48 B
     float *pred = feat + 4 * s->ncells;
-    // the network runs on its own stream: its inputs/outputs live in this sim's scratch
-    cudaError_t e = cudaStreamSynchronize(s->stream);
+    // the network runs on its own stream, its inputs and outputs in this sim's scratch: after the
+    // work on the sim's stream, which then waits for it
+    cudaError_t e = stream_after(mlp_stream(mlp), s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "warm start");
     lbm_status st = lbm_mlp_features(mlp, s->prob.nx, s->prob.ny, kn, u_w, feat);
     if (st == LBM_OK) st = lbm_mlp_forward(mlp, feat, (int)s->ncells, pred);
+    e = stream_after(s->stream, mlp_stream(mlp));
+    if (e != cudaSuccess) cudaStreamSynchronize(mlp_stream(mlp));    // nothing outlives the call
     if (st != LBM_OK) return st;
-    e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(e, "warm start");
     e = launch_warm_state(pred, s->prob.nx, s->prob.ny, s->args.pa, s->args.py, s->vs.m, s->hdr->xi1, s->hdr->w1,
                           u_w / s->u_ref, planar_target(s), s->prob.prec, s->stream);

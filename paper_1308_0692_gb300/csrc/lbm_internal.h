@@ -151,6 +151,21 @@ cudaError_t launch_moments_state(int prec, const double *mom, int nx, int ny, lo
 cudaError_t launch_add_f32(float *y, const float *x, long count, cudaStream_t s);
 cudaError_t launch_widen(const float *src, double *dst, long count, cudaStream_t s);
 
+// Work enqueued on `waiter` from here on runs after what `first` holds now.
+inline cudaError_t stream_after(cudaStream_t waiter, cudaStream_t first)
+{
+    if (waiter == first) return cudaSuccess;
+    cudaEvent_t ev;
+    cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) return e;
+    e = cudaEventRecord(ev, first);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(waiter, ev, 0);
+    cudaEventDestroy(ev);                // released once the work on it is done
+    return e;
+}
+
+struct lbm_mlp;
+cudaStream_t mlp_stream(const lbm_mlp *p);
 // warm start (mlp.cu): h from normalised predicted moments [ncells][6]
 cudaError_t launch_warm_state(const float *pred, int nx, int ny, long pa, long py, int m, const double *xi1,
                               const double *w1, double uw_over_uref, void *h, int prec, cudaStream_t s,

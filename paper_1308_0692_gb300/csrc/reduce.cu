@@ -5,6 +5,7 @@
 #include <cmath>
 
 #include "../../include/lbm.h"
+#include "hermite_state.cuh"
 #include "lbm_internal.h"
 
 namespace {
@@ -388,28 +389,22 @@ __global__ void widen_kernel(const float *src, double *dst, long count)
 // rho' delta_ij)(xi_i xi_j - delta_ij)] with rho' = (rho - 1)/u_ref, j' = rho u / u_ref,
 // P' = (P - I)/u_ref (the inverse of the moment map of lbm_moments on sets exact to degree 4).
 template <typename T>
-__global__ void moments_state_kernel(const double *mom, int nx, long ncells, long pa, long py, int m,
-                                     const TableHeader *hdr, double inv_u_ref, T *h)
+__global__ void moments_state_kernel(const double *mom, int nx, int ny, long pa, long py, int m, const TableHeader *hdr,
+                                     double inv_u_ref, T *h)
 {
-    const long stride = (long)gridDim.x * blockDim.x;
-    for (long c = (long)blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += stride) {
-        const long y = c / nx, co = y * py + (c - y * nx);
-        const double rho = mom[c];
-        const double rp = (rho - 1.0) * inv_u_ref;
-        const double jx = rho * mom[ncells + c] * inv_u_ref, jy = rho * mom[2 * ncells + c] * inv_u_ref;
-        const double pxx = (mom[3 * ncells + c] - 1.0) * inv_u_ref, pxy = mom[4 * ncells + c] * inv_u_ref;
-        const double pyy = (mom[5 * ncells + c] - 1.0) * inv_u_ref;
-        for (int iy = 0; iy < m; ++iy) {
-            const double ey = hdr->xi1[iy];
-            for (int ix = 0; ix < m; ++ix) {
-                const double ex = hdr->xi1[ix];
-                const double v = hdr->w1[ix] * hdr->w1[iy] *
-                                 (rp + ex * jx + ey * jy +
-                                  0.5 * ((pxx - rp) * (ex * ex - 1.0) + 2.0 * pxy * ex * ey + (pyy - rp) * (ey * ey - 1.0)));
-                h[(long)(iy * m + ix) * pa + co] = (T)v;
-            }
-        }
-    }
+    __shared__ double c[LBM_MAX_M][3];
+    hermite::row_table(c, hdr->xi1, hdr->w1, m);
+    const int iy = threadIdx.x >> 5;
+    const long ncells = (long)nx * ny, cell = (long)blockIdx.x * 32 + (threadIdx.x & 31);
+    if (cell >= ncells) return;
+    const double rho = mom[cell];
+    const hermite::Cell q = {(rho - 1.0) * inv_u_ref,
+                             rho * mom[ncells + cell] * inv_u_ref,
+                             rho * mom[2 * ncells + cell] * inv_u_ref,
+                             (mom[3 * ncells + cell] - 1.0) * inv_u_ref,
+                             mom[4 * ncells + cell] * inv_u_ref,
+                             (mom[5 * ncells + cell] - 1.0) * inv_u_ref};
+    hermite::put_row(q, c, hdr->xi1[iy], hdr->w1[iy], iy, m, (int)(cell % nx), (int)(cell / nx), ny, pa, py, h, false);
 }
 
 // planar FP64 [a][c] <-> state of layout (pa, py) and type T
@@ -440,11 +435,11 @@ __global__ void axpy_kernel(float *y, const float *x, long count)
 cudaError_t launch_moments_state(int prec, const double *mom, int nx, int ny, long pa, long py, int m,
                                  const TableHeader *hdr, double u_ref, void *h, cudaStream_t s)
 {
-    const long ncells = (long)nx * ny;
+    const unsigned nb = (unsigned)(((long)nx * ny + 31) / 32);
     if (prec == LBM_FP64)
-        moments_state_kernel<double><<<152 * 8, 256, 0, s>>>(mom, nx, ncells, pa, py, m, hdr, 1.0 / u_ref, (double *)h);
+        moments_state_kernel<double><<<nb, 32 * m, 0, s>>>(mom, nx, ny, pa, py, m, hdr, 1.0 / u_ref, (double *)h);
     else
-        moments_state_kernel<float><<<152 * 8, 256, 0, s>>>(mom, nx, ncells, pa, py, m, hdr, 1.0 / u_ref, (float *)h);
+        moments_state_kernel<float><<<nb, 32 * m, 0, s>>>(mom, nx, ny, pa, py, m, hdr, 1.0 / u_ref, (float *)h);
     return cudaGetLastError();
 }
 
