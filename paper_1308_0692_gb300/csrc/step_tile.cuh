@@ -76,6 +76,13 @@ __global__ void __launch_bounds__(tile_cells<NS>() * NS) step_tile_kernel(const 
     TC hs[RPL * M];
 #pragma unroll
     for (int k = 0; k < RPL * M; ++k) hs[k] = (TC)hp[k * ncells];
+    // the source beside them: read where it is added, its latency stood after the moment exchange
+    [[maybe_unused]] TC sv[SOURCE ? RPL * M : 1];
+    if constexpr (SOURCE) {
+        const TS *hsrc = reinterpret_cast<const TS *>(a.src) + (long)(g * RPL * M) * ncells + c;
+#pragma unroll
+        for (int k = 0; k < RPL * M; ++k) sv[k] = (TC)hsrc[k * ncells];
+    }
 
     // ---- wall densities of the faces this cell touches (Eq. 9) ----
     TC rb = 0, rt = 0, rl = 0, rr = 0;
@@ -239,7 +246,6 @@ __global__ void __launch_bounds__(tile_cells<NS>() * NS) step_tile_kernel(const 
 #pragma unroll
         for (int k = 0; k < RPL * M; ++k) hs[k] *= (TC)a.b;
     TS *hn = reinterpret_cast<TS *>(a.hn) + (long)(g * RPL * M) * ncells + c;
-    const TS *hsrc = SOURCE ? reinterpret_cast<const TS *>(a.src) + (long)(g * RPL * M) * ncells + c : nullptr;
 #pragma unroll
     for (int r = 0; r < RPL; ++r) {
         const int iy = g * RPL + r;
@@ -248,7 +254,7 @@ __global__ void __launch_bounds__(tile_cells<NS>() * NS) step_tile_kernel(const 
         const TC jj = wom * jx;
         auto put = [&](int ix, TC v) {
             const long off = (long)(r * M + ix) * ncells;
-            if (SOURCE) v += (TC)hsrc[off];
+            if constexpr (SOURCE) v += sv[r * M + ix];
             if (ACC) {
                 const TC d = v - (TC)hp[off];
                 psd += d * d;
