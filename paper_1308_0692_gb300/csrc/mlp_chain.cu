@@ -97,6 +97,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == 0) tmem_alloc(&s_tmem, BN);
+    // the kernels of a step are set up while the one before runs and wait for it here
+    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;\n" ::: "memory");
     // layer 0's operand: the four features, zeros up to K = 16
     if (cg == 0) {
         float f[4] = {0.f, 0.f, 0.f, 0.f};
@@ -295,8 +297,8 @@ cudaError_t prepare_chain()
 cudaError_t launch_chain(bool train, const ChainMaps &maps, const ChainArgs &a, cudaStream_t s)
 {
     const int grid = 2 * ((a.M + ROWS - 1) / ROWS);
-    if (train) mlp_chain_kernel<true><<<grid, THREADS, SMEM, s>>>(maps, a);
-    else mlp_chain_kernel<false><<<grid, THREADS, SMEM, s>>>(maps, a);
+    if (train) return launch_after(mlp_chain_kernel<true>, dim3(grid), THREADS, SMEM, s, maps, a);
+    mlp_chain_kernel<false><<<grid, THREADS, SMEM, s>>>(maps, a);     // a single launch: nothing to overlap
     return cudaGetLastError();
 }
 

@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(256, 1)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == 0) tmem_alloc(&s_tmem, 128);
+    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;\n" ::: "memory");
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(256) mlp_reduce_adam_kernel(const __grid_const
     constexpr int LDQ[NL] = {PADW[0], PADW[1], PADW[2], PADW[3]}, LDT[NL] = {PADW[1], PADW[2], PADW[3], PADW[4]};
     __shared__ float tile[32][33];
     const int bid = blockIdx.x;
+    asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;\n" ::: "memory");
     if (bid >= B.first[NL]) {
         // biases: the row tiles' column sums, 32 columns a block, 8 groups of tiles in turn, then
         // the groups in order
@@ -248,15 +250,14 @@ cudaError_t prepare_grads() { return cudaFuncSetAttribute(mlp_grad_kernel, cudaF
 
 cudaError_t launch_grads(const GradMaps &maps, int ktiles, int splits, float *part, int *status, cudaStream_t s)
 {
-    mlp_grad_kernel<<<dim3(WTILES, splits), 256, SMEM, s>>>(maps, ktiles, (ktiles + splits - 1) / splits, part, status);
-    return cudaGetLastError();
+    return launch_after(mlp_grad_kernel, dim3(WTILES, splits), 256, SMEM, s, maps, ktiles, (ktiles + splits - 1) / splits, part,
+                        status);
 }
 
 cudaError_t launch_reduce_adam(const AdamArgs &a, cudaStream_t s)
 {
     const int blocks = weight_blocks().first[NL] + (BIASES + 31) / 32;
-    mlp_reduce_adam_kernel<<<blocks, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(mlp_reduce_adam_kernel, dim3(blocks), 256, 0, s, a);
 }
 
 }  // namespace mlpk

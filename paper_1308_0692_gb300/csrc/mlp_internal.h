@@ -51,6 +51,24 @@ struct AdamArgs {
     float lr, c1, c2;          // step size, 1 - beta^t
 };
 
+// Launch as a programmatic dependent of the stream's last kernel (the kernels of this network wait
+// for it themselves); a plain launch on the legacy stream.
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*fn)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, const A &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = s != nullptr ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, args...);
+}
+
 cudaError_t prepare_chain();
 cudaError_t launch_chain(bool train, const ChainMaps &maps, const ChainArgs &a, cudaStream_t s);
 cudaError_t prepare_grads();
