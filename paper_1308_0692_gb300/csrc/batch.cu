@@ -32,7 +32,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_internal.h"
-#include "step_wall.cuh"
+#include "step_kernel.cuh"
 
 lbm_status lbm_norms_fail(lbm_status s, const char *msg);
 

@@ -9,14 +9,14 @@
 // and exact relaxation (relaxation factor exp(-omega) on the stored half-relaxed state,
 // set by the host), the steady state converges at second order in the grid spacing.
 //
-// Same decomposition as step_wall.cuh (32-cell segments, G warps per segment owning M/G
+// Same decomposition as step_kernel.cuh (32-cell segments, G warps per segment owning M/G
 // velocity rows, moments through shared memory, wall segments in a second kernel), with
 // register loads of the two upwind neighbours per direction.  TILED: the state is the
 // strip-tiled FP32 layout of the column march (lbm_internal.h); the kernel then serves as
 // the wall kernel beside the second-order march (step_so_march.cu).
 #pragma once
 
-#include "step_wall.cuh"
+#include "step_kernel.cuh"
 
 namespace lbmk {
 

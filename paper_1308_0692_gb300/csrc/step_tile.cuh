@@ -29,7 +29,7 @@
 
 #include <type_traits>
 
-#include "step_wall.cuh"
+#include "step_kernel.cuh"
 
 namespace lbmk {
 

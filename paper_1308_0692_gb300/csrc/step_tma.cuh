@@ -18,7 +18,7 @@
 
 #include <cstdint>
 
-#include "step_wall.cuh"
+#include "step_kernel.cuh"
 
 namespace lbmk {
 
