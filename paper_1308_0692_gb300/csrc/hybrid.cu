@@ -703,18 +703,25 @@ __device__ __forceinline__ void plain_tiles(const PlainArgs<TC> &p, const int2 *
 // evenly, else two; a full-range tile (N nodes) takes one warp
 __host__ __device__ constexpr int half_warps(int n) { return (2 * n) % 4 == 0 ? 4 : 2; }
 
-// One step, one launch: the blocks for the interface cells first (one warp per cell: their
-// projections are long latency chains), then those for the half-range and the full-range
-// tiles, so that all three run side by side.
+// One step, one launch: blocks for the interface cells (one warp per cell: their projections are
+// long latency chains) and for the half-range and the full-range tiles.  Where the grid is more
+// than a few blocks per SM, interface blocks alternate with tile blocks: dealt first they fill
+// the chip for their whole latency with the FP64 or load units half idle.  Measured, us a step,
+// first / alternating: 256^2 N = 4, 16-cell ring FP64 49.7 / 49.0, FP32 15.1 / 13.1; 512^2 134.9 /
+// 129.2 and 23.9 / 22.0; 200^2 N = 6, 8 cells 79.3 / 76.8 and 27.9 / 24.9, N = 3 FP32 13.3 / 10.1;
+// one in three or four the same but 512^2 FP32 (23.8).  A grid that is in flight almost at once
+// starts its longest chains first: 128^2 N = 4, 4 cells FP64 27.4 / 28.3.
 struct StepLists {
     const int *cells;          // interface cells
     int ncells;
     const int2 *tiles[2];      // half-range, full-range tiles with a plain cell
     int ntiles[2];
+    int every;                 // one block in `every` takes interface cells, until they are dealt (1 or 2)
 };
 
 // blocks a SM the FP32 build asks for: eight (64 registers a thread) where that does not
-// spill, six for the 100- and 144-velocity half-range sets; FP64 as the compiler chooses
+// spill, six for the 100- and 144-velocity half-range sets; FP64 as the compiler chooses (four of
+// 128 registers for N = 4: 512^2 129.2 to 121.9 us a step, but 256^2 49.0 to 51.1, 128^2 27.4 to 30.0)
 template <int N, typename TS>
 constexpr int hybrid_min_blocks() { return sizeof(TS) == 8 ? 1 : (N >= 5 ? 6 : 8); }
 
@@ -735,7 +742,10 @@ __global__ void __launch_bounds__(32 * HWARPS, hybrid_min_blocks<N, TS>()) hybri
     // the next step's blocks are set up while this one runs (for the interface cells with the
     // projection matrices in shared memory) and wait for it before they read the state
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    if (IfShared<N, TS>::STAGED && bid < ifb) {
+    const bool interface = bid < ifb * L.every && bid % L.every == 0;
+    // block among the interface blocks, or among the others
+    const int k0 = interface ? bid / L.every : bid - min(ifb, bid / L.every + 1);
+    if (IfShared<N, TS>::STAGED && interface) {
         const HybTabT<TS> &tb = *static_cast<const HybTabT<TS> *>(a.tab);
         for (int k = threadIdx.x; k < 4 * N * N * N * N; k += 32 * HWARPS) {
             u.sh.pt[0][k] = tb.pt[0][k];
@@ -744,13 +754,13 @@ __global__ void __launch_bounds__(32 * HWARPS, hybrid_min_blocks<N, TS>()) hybri
         __syncthreads();
     }
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    if (bid < ifb) {
-        const int wi = threadIdx.x >> 5, ci = bid * HWARPS + wi;
+    if (interface) {
+        const int wi = threadIdx.x >> 5, ci = k0 * HWARPS + wi;
         if (ci < L.ncells) interface_cell<N, TS>(a, u.sh, wi, L.cells[ci], resid);    // whole warps
-    } else if (bid < ifb + hbk) {
-        plain_tiles<2 * N, GH>(ph, L.tiles[0], L.ntiles[0], bid - ifb, resid, u.hx);
+    } else if (k0 < hbk) {
+        plain_tiles<2 * N, GH>(ph, L.tiles[0], L.ntiles[0], k0, resid, u.hx);
     } else {
-        plain_tiles<N, 1>(pf, L.tiles[1], L.ntiles[1], bid - ifb - hbk, resid, u.fx);
+        plain_tiles<N, 1>(pf, L.tiles[1], L.ntiles[1], k0 - hbk, resid, u.fx);
     }
 }
 
@@ -759,9 +769,12 @@ cudaError_t launch_step_n(const HybArgs &a, const PlainArgs<TS> &ph, const Plain
                           int resid, cudaStream_t st)
 {
     constexpr int GH = half_warps(N);
-    const int blocks = (L.ncells + HWARPS - 1) / HWARPS + (L.ntiles[0] + HWARPS / GH - 1) / (HWARPS / GH) +
-                       (L.ntiles[1] + HWARPS - 1) / HWARPS;
+    const int ifb = (L.ncells + HWARPS - 1) / HWARPS;
+    const int others = (L.ntiles[0] + HWARPS / GH - 1) / (HWARPS / GH) + (L.ntiles[1] + HWARPS - 1) / HWARPS;
+    const int blocks = ifb + others;
     if (blocks == 0) return cudaSuccess;
+    StepLists D = L;
+    D.every = blocks >= 4 * 152 && others >= ifb ? 2 : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(32 * HWARPS);
@@ -771,7 +784,7 @@ cudaError_t launch_step_n(const HybArgs &a, const PlainArgs<TS> &ph, const Plain
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = st != nullptr ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, hybrid_step_kernel<N, TS>, a, ph, pf, L, resid);
+    return cudaLaunchKernelEx(&cfg, hybrid_step_kernel<N, TS>, a, ph, pf, D, resid);
 }
 
 template <typename TS>
