@@ -154,9 +154,14 @@ cudaError_t launch_widen(const float *src, double *dst, long count, cudaStream_t
 // Work enqueued on `waiter` from here on runs after what `first` holds now.
 inline cudaError_t stream_after(cudaStream_t waiter, cudaStream_t first)
 {
-    if (waiter == first) return cudaSuccess;
+    // the callers end with a synchronisation: a stream under capture is refused before the capture
+    // takes the other stream in
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(first, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+    if (e != cudaSuccess || waiter == first) return e;
     cudaEvent_t ev;
-    cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e != cudaSuccess) return e;
     e = cudaEventRecord(ev, first);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(waiter, ev, 0);
