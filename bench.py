@@ -545,7 +545,7 @@ FP64_SO_OPS_WALL = 24.0
 
 # FP64 pipe instructions (lane operations) per node-velocity update of the FP64 step, from the
 # ncu count of sm__inst_executed_pipe_fp64 on the 1024^2 x 144 FP64 step (profiles/)
-FP64_PIPE_OPS_PER_UPDATE = 10.1
+FP64_PIPE_OPS_PER_UPDATE = 7.58
 
 
 # refinement design behind the time-to-residual headline: "per_instance" (one simulation per

@@ -410,7 +410,9 @@ void fill_args(lbm_sim *s, const TableHeader &hdr)
 
 // Velocity slices and cells of a block of step_tile.cuh (load paths 0 and 1, the correction
 // march; dp: FP64 arithmetic, the FP64 march and the defect pass).  Measured over 19 grids
-// (1 x 100 to 512 x 512, M = 3 to 12; us per step, replayed graphs):
+// (1 x 100 to 512 x 512, M = 3 to 12; us per step, replayed graphs; both sides with the build
+// that the line was drawn with, the kernel has since gained 5 to 10 %: now M = 8 FP64 128^2 23.6,
+// 192^2 44.4, FP32 128^2 3.9, 333 x 251 10.1, M = 12 FP64 300^2 205, 512^2 556):
 //   FP64 is bound by the FP64 pipe of each SM quarter, so small blocks that spread evenly win,
 //     with one velocity row a thread while the grid leaves the quarters short of warps (M = 8:
 //     64^2 12.1 against 15.6 with two rows, 128^2 25.2 against 28.1) and two or three rows a
