@@ -422,23 +422,32 @@ void fill_args(lbm_sim *s, const TableHeader &hdr)
 //     128^2 4.8; 32 places 5.9, one row a thread 6.0), 32 places where there are enough of
 //     them to fill the chip (333 x 251 10.4 against 10.8), few cells with one row a thread
 //     (40 x 33 2.9 against 3.2); small sets whole rows a thread (M = 4: 128^2 2.7 against 2.9).
+// Beyond the L2 (two states of more than 129 MB together) narrow blocks fetch lines they use half of
+// and find fewer of the y neighbours in the L1: 32 places, and from 2M cells on two rows of cells, at 1000 x
+// 900 and 2047 x 1500 M = 12 FP32 384 to 241 and 1797 to 861 (six slices of 16 places; 331 to 336 and
+// 650 to 580 from four of 32 to two of 32 x 2 at 1.2M and 2.1M cells), M = 8 395 to 339 at 2047 x 1500,
+// M = 3 29.1 to 15.2 and 98.0 to 51.9.  FP64 with small sets takes whole rows a thread once the quarters
+// have warps enough: M = 4 at 200^2, 300 x 250, 600^2 16.5 / 24.1, 27.4 / 26.3, 118 / 98 (four slices /
+// one), M = 6 at 300 x 250, 400 x 300, 600^2 51.5 / 51.8, 79.2 / 77.8, 224 / 209 (six / two).
 struct TilePlan {
     int ns, w, r;
 };
 
 TilePlan tile_plan(bool dp, int m, long ncells)
 {
-    if (m == 3) return {1, 16, 2};
+    const bool large = ncells >= 2000000;
     if (dp) {
-        if (m == 4) return {4, 8, 1};
-        if (m == 6) return {6, 8, 2};
+        if (m == 3) return {1, 16, 2};
+        if (m == 4) return ncells < 60000 ? TilePlan{4, 8, 1} : TilePlan{1, 8, 4};
+        if (m == 6) return ncells < 100000 ? TilePlan{6, 8, 2} : TilePlan{2, 8, 2};
         if (m == 8) return ncells < 25000 ? TilePlan{8, 4, 1} : TilePlan{4, 8, 1};
         return ncells < 100000 ? TilePlan{12, 8, 1} : TilePlan{4, 8, 1};
     }
+    if (m == 3) return ncells < 20000 ? TilePlan{1, 16, 2} : TilePlan{1, 32, 2};
     if (m == 4) return ncells < 4000 ? TilePlan{4, 16, 2} : ncells < 50000 ? TilePlan{1, 16, 2} : TilePlan{1, 32, 2};
-    if (m == 6) return ncells < 20000 ? TilePlan{6, 8, 2} : TilePlan{2, 32, 1};
-    if (m == 8) return ncells < 2500 ? TilePlan{8, 8, 1} : ncells < 50000 ? TilePlan{4, 16, 1} : TilePlan{4, 32, 1};
-    return {6, 16, 1};
+    if (m == 6) return ncells < 20000 ? TilePlan{6, 8, 2} : TilePlan{2, 32, large ? 2 : 1};
+    if (m == 8) return ncells < 2500 ? TilePlan{8, 8, 1} : ncells < 50000 ? TilePlan{4, 16, 1} : TilePlan{4, 32, large ? 2 : 1};
+    return ncells < 30000 ? TilePlan{6, 16, 1} : large ? TilePlan{2, 32, 2} : TilePlan{4, 32, 1};
 }
 
 // Longest one-column channel whose steps run together on a cluster (step_column.cu): beyond, the
@@ -448,8 +457,18 @@ TilePlan tile_plan(bool dp, int m, long ncells)
 // 2.7 / 2.6; M = 12 at 320, 500 2.9 / 3.8, 3.9 / 3.8.
 int column_cells(bool dp, int m) { return m == 12 ? (dp ? 300 : 450) : m == 8 ? 450 : 512; }
 
-// the same for slices the caller chose (lbm_set_variant)
-TilePlan tile_plan_for(bool dp, int ns) { return dp ? TilePlan{ns, 8, ns == 1 ? 4 : 1} : TilePlan{ns, ns >= 6 ? 16 : 32, ns == 1 ? 2 : 1}; }
+// The same for slices the caller chose (lbm_set_variant): the plan's shape where it has as many, else
+// 32 places in FP32, and in FP64 the fewest cells that fill a warp or two evenly (M = 8, two slices,
+// 600^2: 8 places 687 us a step, 8 x 2 354; M = 12, three slices 8 places 1007, 8 x 4 805, six
+// slices 8 places 992, 16 places 759).
+TilePlan tile_plan_for(bool dp, int m, long ncells, int ns)
+{
+    const TilePlan t = tile_plan(dp, m, ncells);
+    if (t.ns == ns) return t;
+    if (!dp) return {ns, 32, ns == 1 ? 2 : 1};
+    if (ns == 6) return {6, 16, 1};
+    return {ns, 8, ns == 1 || ns == 3 ? 4 : ns == 2 ? 2 : 1};
+}
 
 int grid_for(long ncells, int lanes)
 {
@@ -599,7 +618,7 @@ lbm_status set_lanes(lbm_sim *s, int lanes)
     s->nparts_step = s->grid + wall_grid(lanes, (int)segs.size());
     if (s->order == 1 && s->prefetch <= 1) {
         const bool dp = s->prob.prec == LBM_FP64;
-        const TilePlan t = s->lanes_set ? tile_plan_for(dp, lanes) : tile_plan(dp, s->vs.m, s->ncells);
+        const TilePlan t = s->lanes_set ? tile_plan_for(dp, s->vs.m, s->ncells, lanes) : tile_plan(dp, s->vs.m, s->ncells);
         s->slices = t.ns;
         s->args.tile_w = t.w;
         s->args.tile_r = t.r;
