@@ -349,7 +349,7 @@ __device__ void interface_cell(const HybArgs &a, IfShared<N, TS> &sh, int wi, in
             if (f >= 2 || a.cavity) wall_ghost(a, S, hc, f < 2 ? f + 2 : f - 2, nbv[f]);
         } else if (set_of[f] != sj) {
             nbv[f] = sh.seen[wi][f];
-            if (sizeof(T) == 8)
+            if (sizeof(T) == 8 || N <= 4)
                 project_part(tb, pt[set_of[f]], set_of[f], sh.raw[wi][f], tb.away[sj][f >> 1][f & 1],
                              tb.naway[sj][f >> 1][f & 1], nbv[f]);
             else
