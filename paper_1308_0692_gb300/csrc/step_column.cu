@@ -37,6 +37,8 @@ __device__ __forceinline__ unsigned peer(const void *p, unsigned rank)
     asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
     return r;
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 __device__ __forceinline__ void put(unsigned at, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;\n" ::"r"(at), "d"(v) : "memory"); }
 __device__ __forceinline__ void put(unsigned at, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(at), "f"(v) : "memory"); }
 
@@ -80,6 +82,7 @@ template <typename T, int M>
 __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ StepArgs a, int nc, int steps, int resid)
 {
     using Sh = Shape<M>;
+    cluster_arrive();                              // waited for before the first write into a neighbour
     constexpr int P = Sh::P, V = Sh::V, S = Sh::S, HALF = Sh::HALF, GS = Sh::GS, NG = Sh::NG, NV = M * M;
     constexpr bool DP = sizeof(T) == 8;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -152,7 +155,8 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
                 for (int k = 0; k < V; ++k) put(above + b * flip + k * (unsigned)sizeof(T), h[k]);
         }
         __syncwarp();
-        asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+        cluster_arrive();
+        cluster_wait();
     };
     // sums over a cell's threads of v, xi_x v and the two halves of xi_y v
     auto sums = [&](const T (&v)[V], T &rho, T &jx, double &jd, double &ju) {
@@ -202,6 +206,8 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
     double jd, ju;
     sums(h, rho, jx, jd, ju);
     if (wall) rho_w = (T)((up ? -jd : ju) * a.inv_dy_wall);
+    __syncwarp();
+    cluster_wait();                                // every CTA of the cluster runs: its shared memory may be written
     publish(0);
     T psd = 0, psn = 0;
     for (int n = 0; n < steps; ++n) {
@@ -271,7 +277,8 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
     }
     // no CTA leaves while a neighbour may still write into it
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 
 template <typename T, int M>
