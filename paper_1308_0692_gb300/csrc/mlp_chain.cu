@@ -173,10 +173,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
         if (i != 3) {
             tmem_ld32(lanes + (uint32_t)(cg * 32), v);
             if (fwd) {
-                const float *bias = p.b[i];
+                const float *bias = p.b[i];            // (no read-only path: the step before updates them while this grid is set up)
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
-                    const float zj = v[j] + __ldg(bias + n0 + j), e = gelu_e(zj);
+                    const float zj = v[j] + bias[n0 + j], e = gelu_e(zj);
                     if (TRAIN) {
                         z[TRAIN ? j : 0] = zj;
                         gp[TRAIN ? j : 0] = e;
@@ -205,7 +205,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
             const float scale = 2.0f / ((float)p.M * 6.0f);
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
-                y[c] += __ldg(p.b[3] + c);
+                y[c] += p.b[3][c];
                 if (!TRAIN) {
                     if (valid && rank == 0) p.y[grow * 6 + c] = y[c];
                 } else if (valid) {

@@ -26,3 +26,12 @@ def test_column_kernel_waits_for_its_cluster_before_the_first_remote_store():
     straight = re.sub(r"^ {4}auto \w+ = \[&\].*?^ {4}\};", "", body[:first], flags=re.M | re.S)   # less the lambdas' bodies
     arrive, wait = straight.find("cluster_arrive();"), straight.find("cluster_wait();")
     assert 0 <= arrive < wait
+
+
+def test_training_kernels_take_no_read_only_loads():
+    """The kernels of a training step are programmatic dependents of each other: the one that writes
+    a parameter still runs when the one that reads it starts.  The read-only path is for data that
+    nobody writes during a kernel."""
+    for name in ("mlp_chain.cu", "mlp_grad.cu"):
+        src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        assert not re.search(r"__ldg|ld\.global\.nc|__restrict__", src), name
