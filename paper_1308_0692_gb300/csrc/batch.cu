@@ -202,11 +202,12 @@ __device__ __forceinline__ ItemAddr load_addr(const BatchItem *items, long nitem
 // separate from the lean wall-free path so that the latter keeps a small register
 // footprint.  The item's addressing `A` was fetched one group earlier; its coefficients and
 // the instance's convergence flag are fetched here together with the state.  A segment of
-// an instance that converged since the item list was built is read but not written.  All
-// threads of the block call it together (shared-memory exchanges inside).
+// an instance that converged since the item list was built is read but not written.  The state
+// comes by ordinary loads: the same launch wrote it in the step before (never the read-only path).
+// All threads of the block call it together (shared-memory exchanges inside).
 template <typename TS, typename TC, int M, int G, bool WALLS, int MODE>
 __device__ __forceinline__ void batch_group(const BatchArgs &a, const BatchItem *items, long grp,
-                                            const ItemAddr &A, long s, const TS *__restrict__ h,
+                                            const ItemAddr &A, long s, const TS *h,
                                             TS *__restrict__ hn, bool resid,
                                             TC (&s_mom)[3][G][lbmk::Shape<G>::SPB][32],
                                             double (&s_wall)[4][G][lbmk::Shape<G>::SPB][32])
@@ -296,7 +297,7 @@ __device__ __forceinline__ void batch_group(const BatchArgs &a, const BatchItem 
                     for (int k = lane; k < NSIDE; k += 32) {
                         const int r = k / HALF, q = k - r * HALF;
                         const int iy = g * RPL + r, ix = side == 0 ? q : M - HALF + q;
-                        const TC v = (TC)__ldg(hi + vo(iy * M + ix) + cL);
+                        const TC v = (TC)hi[vo(iy * M + ix) + cL];
                         const TC xv = pk<TC>(a.xi, a.xi_f, ix) * v;
                         part += side == 0 ? -(double)xv : (double)xv;
                     }
@@ -316,7 +317,7 @@ __device__ __forceinline__ void batch_group(const BatchArgs &a, const BatchItem 
                 TC rowsum = 0, left = 0, right = 0;
 #pragma unroll
                 for (int ix = 0; ix < M; ++ix) {
-                    const TC v = (TC)__ldg(hi + vo(iy * M + ix) + c_at);
+                    const TC v = (TC)hi[vo(iy * M + ix) + c_at];
                     rowsum += v;
                     if (ix < HALF) left -= pk<TC>(a.xi, a.xi_f, ix) * v;
                     if (ix >= M - HALF) right += pk<TC>(a.xi, a.xi_f, ix) * v;
@@ -367,7 +368,7 @@ __device__ __forceinline__ void batch_group(const BatchArgs &a, const BatchItem 
 #pragma unroll
             for (int ix = 0; ix < M; ++ix) {
                 const TS *hp = hi + vo(iy * M + ix);
-                const TC hc = (TC)__ldg(hp + c_at);
+                const TC hc = (TC)hp[c_at];
                 const TC xix = pk<TC>(a.xi, a.xi_f, ix);
                 TC v = hc;
                 if (ix >= M - HALF || ix < HALF) {
@@ -375,14 +376,14 @@ __device__ __forceinline__ void batch_group(const BatchArgs &a, const BatchItem 
                     if (WALLS && (ix >= M - HALF ? wl : wr))
                         hx = pk<TC>(a.w1, a.w1_f, ix) * wy * (ix >= M - HALF ? rl_t : rr_t);
                     else
-                        hx = (TC)__ldg(hp + (ix >= M - HALF ? c_left : c_right));
+                        hx = (TC)hp[ix >= M - HALF ? c_left : c_right];
                     v += (xix < TC(0) ? -xix : xix) * cx * (hx - hc);
                 }
                 TC hy;
                 if (WALLS && ywall)
                     hy = pk<TC>(a.w1, a.w1_f, ix) * wy * (rho_y * (TC(1) + xix * u_y) + xix * drive_y);
                 else
-                    hy = (TC)__ldg(hp + cy_idx);
+                    hy = (TC)hp[cy_idx];
                 v += nuy * (hy - hc);
                 hs[r * M + ix] = v;
                 R += v;
@@ -423,7 +424,7 @@ __device__ __forceinline__ void batch_group(const BatchArgs &a, const BatchItem 
                 if (MODE == BATCH_CORRECT) v += (TC)__ldg(a.src + A.off + off);
                 TC d = 0;
                 if (resid) {
-                    d = v - (TC)__ldg(hi + off);
+                    d = v - (TC)hi[off];
                     psd += d * d;
                     psn += v * v;
                 }
@@ -455,7 +456,7 @@ __global__ void __launch_bounds__(lbmk::Shape<G>::THREADS, 2) batch_kernel(const
 
     for (int si = 0; si < a.nsteps; ++si) {
         const long s = a.step0 + si;
-        const TS *__restrict__ h = reinterpret_cast<const TS *>(a.buf[s & 1]);
+        const TS *h = reinterpret_cast<const TS *>(a.buf[s & 1]);
         TS *__restrict__ hn = reinterpret_cast<TS *>(a.buf[(s + 1) & 1]);
         const bool resid = MODE == BATCH_DEFECT || ((s + 1) % a.resid_every) == 0;
         // wall-free segments, then segments with wall cells, both round-robin over the blocks;

@@ -35,3 +35,13 @@ def test_training_kernels_take_no_read_only_loads():
     for name in ("mlp_chain.cu", "mlp_grad.cu"):
         src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
         assert not re.search(r"__ldg|ld\.global\.nc|__restrict__", src), name
+
+
+def test_batch_segment_kernel_takes_no_read_only_loads_of_the_state():
+    """A launch takes many steps: what it reads in one it has written, from other multiprocessors,
+    in the step before."""
+    body = _body("batch.cu", "batch_group")
+    loads = re.findall(r"__ldg\(([^;]*);", body)
+    assert loads and all(re.match(r"p\)|p \+ 1\)|a\.src", x) for x in loads), loads
+    src = open(os.path.join(CSRC, "batch.cu")).read()
+    assert not re.search(r"const TS \*__restrict__ h\b", src)
