@@ -12,10 +12,12 @@
 //     cluster barrier a step;
 //   * transport: a0 h + nu h_up with the neighbour's value, or at a wall G1 rho_w + G0 with the
 //     ghost's coefficients (Eq. 8) in the places of nu and zero: no extra operations;
-//   * the moments, and the momentum leaving through each wall (the down- and up-moving halves of
-//     j_y), as sums over the cell's threads in two stages of at most four terms;
-//   * the next rho_w (Eq. 9) from those sums: the row sums of the relaxed state are
-//     R_iy + omega w_iy (rho + xi_iy j_y).
+//   * the moments as sums over the cell's threads in two stages of at most four terms;
+//   * rho_w (Eq. 9) from the row sums of the state itself, which the wall cells' threads leave in
+//     shared memory before the step's barrier: the same bits wherever a launch begins.  (A recurrence
+//     from the sums of the step before, which made the last bits depend on how the steps were dealt
+//     to calls, took as long: 100 cells, M = 8, FP64 2.88 us a step against 2.80, FP32 1.55
+//     against 1.51.)
 // FP32 keeps the wall sums in FP64, as the other FP32 kernels do.
 #include <cstring>
 
@@ -75,7 +77,7 @@ __host__ __device__ constexpr size_t column_smem(int nc)
 {
     using Sh = Shape<M>;
     return sizeof(T) * ((size_t)2 * (nc + 2) * M * M + (size_t)nc * (2 * Sh::S + 2 * Sh::NG + 2)) +
-           sizeof(double) * ((size_t)nc * (Sh::S + Sh::NG + 2) + 64 + 1);
+           sizeof(double) * ((size_t)nc * (Sh::S + Sh::NG + 1) + 64 + 1);
 }
 
 template <typename T, int M>
@@ -88,12 +90,13 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
     extern __shared__ __align__(16) unsigned char smem[];
     double *const s_j = reinterpret_cast<double *>(smem);            // [nc][S]
     double *const s_jg = s_j + (size_t)nc * S;                       // [nc][NG]
-    double *const s_jt = s_jg + (size_t)nc * NG;                     // [nc][2]: down, up
-    double *const s_red = s_jt + (size_t)nc * 2;                     // [2][32]
+    double *const s_jt = s_jg + (size_t)nc * NG;                     // [nc]
+    double *const s_red = s_jt + nc;                                 // [2][32]
     T *const s_v = reinterpret_cast<T *>(s_red + 64);                // [2][nc + 2][NV]
     T *const s_m = s_v + (size_t)2 * (nc + 2) * NV;                  // [2][nc][S]
     T *const s_mg = s_m + (size_t)2 * nc * S;                        // [2][nc][NG]
     T *const s_mt = s_mg + (size_t)2 * nc * NG;                      // [nc][2]
+    __shared__ double s_out[2][M];                                   // |xi_y| R of the bottom and the top cell's rows
     unsigned rank;
     asm("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
     const int ny = a.ny, y0 = (int)rank * nc, nloc = max(0, min(nc, ny - y0));
@@ -119,17 +122,8 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
             c0[k] = wall ? (T)(f * (wa * (a.xi[ix] * u * a.inv_u_ref))) : T(0);
         }
     }
-    // Eq. 9 after relaxation: sum over the leaving rows of |xi| times their row sums
-    double cA = 0.0, cB = 0.0, W1 = 0.0;
-#pragma unroll
-    for (int i = 0; i < M; ++i) W1 += a.w1[i];
-#pragma unroll
-    for (int i = 0; i < HALF; ++i) {
-        const double o = DP ? a.omw[i] : (double)a.omega_f * (double)a.w1_f[i];
-        cA -= a.xi[i] * o * W1 * a.inv_dy_wall;
-        cB += a.xi[i] * a.xi[i] * o * W1 * a.inv_dy_wall;
-    }
-    const double kJ = (DP ? (a.fold ? 1.0 : a.b) : (double)a.b_f) * a.inv_dy_wall, sB = up ? -cB : cB;
+    const bool edge = on && (y == 0 || y == ny - 1);
+    const double out = fabs(a.xi[iy]) * a.inv_dy_wall;
     const T xo = omw * xiy;
     T rho_w = 0;
     const unsigned below = rank > 0 && act && cl == 0 && on && down ? peer(s_v + ((size_t)(nc + 1) * NV + iy * M + k0), rank - 1) : 0;
@@ -158,8 +152,17 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
         cluster_arrive();
         cluster_wait();
     };
-    // sums over a cell's threads of v, xi_x v and the two halves of xi_y v
-    auto sums = [&](const T (&v)[V], T &rho, T &jx, double &jd, double &ju) {
+    // what the wall cells' rows carry towards a wall, before the barrier; behind it, Eq. 9
+    auto leave = [&] {
+        if (__any_sync(0xffffffffu, edge)) {
+            double p = out * (double)tree<V, T>([&](int k) { return h[k]; });
+            if (P == 2) p += __shfl_xor_sync(0xffffffffu, p, 1);
+            if (edge && k0 == 0) s_out[y == 0 ? 0 : 1][iy] = p;
+        }
+    };
+    auto density = [&] { return (T)tree<HALF, double>([&](int i) { return s_out[up ? 0 : 1][up ? i : M - HALF + i]; }); };
+    // sums over a cell's threads of v, xi_x v and xi_y v
+    auto sums = [&](const T (&v)[V], T &rho, T &jx, T &jy) {
         const T R = tree<V, T>([&](int k) { return v[k]; });
         const T X = tree<V, T>([&](int k) { return xi[k] * v[k]; });
         if (act) {
@@ -173,10 +176,7 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
             if (GS == 1) {                         // three threads a cell: no first stage
                 if (s == 0) s_mt[cl * 2] = s_m[cl * S] + s_m[cl * S + 1] + s_m[cl * S + 2];
                 if (s == 1) s_mt[cl * 2 + 1] = s_m[(nc + cl) * S] + s_m[(nc + cl) * S + 1] + s_m[(nc + cl) * S + 2];
-                if (s == 2) {
-                    s_jt[cl * 2] = s_j[cl * S];
-                    s_jt[cl * 2 + 1] = s_j[cl * S + 2];
-                }
+                if (s == 2) s_jt[cl] = s_j[cl * S] + s_j[cl * S + 2];
             } else if (q < 2) {
                 const T *p = s_m + (size_t)(q * nc + cl) * S + g * GS;
                 s_mg[(q * nc + cl) * NG + g] = tree<GS, T>([&](int k) { return p[k]; });
@@ -190,22 +190,18 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
             if (act && s < 2) {
                 const T *p = s_mg + (size_t)(s * nc + cl) * NG;
                 s_mt[cl * 2 + s] = tree<NG, T>([&](int k) { return p[k]; });
-            } else if (act && s < 4) {
-                const double *p = s_jg + (size_t)cl * NG + (s - 2) * (NG / 2);
-                s_jt[cl * 2 + s - 2] = tree<(NG + 1) / 2, double>([&](int k) { return p[k]; });
+            } else if (act && s == 2) {
+                const double *p = s_jg + (size_t)cl * NG;
+                s_jt[cl] = tree<NG, double>([&](int k) { return p[k]; });
             }
             __syncthreads();
         }
         rho = act ? s_mt[cl * 2] : T(0);
         jx = act ? s_mt[cl * 2 + 1] : T(0);
-        jd = act ? s_jt[cl * 2] : 0.0;
-        ju = act ? s_jt[cl * 2 + 1] : 0.0;
+        jy = act ? (T)s_jt[cl] : T(0);
     };
 
-    T rho, jx;
-    double jd, ju;
-    sums(h, rho, jx, jd, ju);
-    if (wall) rho_w = (T)((up ? -jd : ju) * a.inv_dy_wall);
+    leave();
     __syncwarp();
     cluster_wait();                                // every CTA of the cluster runs: its shared memory may be written
     publish(0);
@@ -213,6 +209,7 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
     for (int n = 0; n < steps; ++n) {
         const int b = n & 1;
         const T *nb = s_v + ((size_t)b * (nc + 2) + (act ? (up ? cl : down ? cl + 2 : cl + 1) : 0)) * NV + iy * M + k0;
+        if (wall) rho_w = density();
         T v[V];
 #pragma unroll
         for (int k = 0; k < V; ++k) {
@@ -224,12 +221,8 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
                 v[k] = h[k] + nuy * (op - h[k]);
             }
         }
-        sums(v, rho, jx, jd, ju);
-        const T jy = (T)(jd + ju);
-        if (wall) {
-            const double out = up ? -jd : ju;
-            rho_w = (T)((sB * jd + sB * ju) + (kJ * out + cA * (double)rho));
-        }
+        T rho, jx, jy;
+        sums(v, rho, jx, jy);
         const T q = DP ? omw * rho + xo * jy : omw * (rho + xiy * jy), jj = omw * jx;
         const bool last = resid && n == steps - 1;
 #pragma unroll
@@ -248,7 +241,10 @@ __global__ void __launch_bounds__(1024) column_kernel(const __grid_constant__ St
             }
             h[k] = o;
         }
-        if (n + 1 < steps) publish(b ^ 1);
+        if (n + 1 < steps) {
+            leave();
+            publish(b ^ 1);
+        }
     }
     T *dst = static_cast<T *>(a.hn) + (size_t)(iy * M + k0) * plane + y;
     if (on)
