@@ -452,10 +452,11 @@ TilePlan tile_plan(bool dp, int m, long ncells)
 
 // Longest one-column channel whose steps run together on a cluster (step_column.cu): beyond, the
 // cluster's 16 SMs take longer than the launches of step_tile.cuh over all of them.  Measured, us
-// per step, cluster / tiles: FP64 M = 8 at 100, 320, 500 cells 2.9 / 6.7, 4.7 / 6.5, 6.9 / 6.3;
-// M = 12 at 200, 320 6.1 / 8.5, 8.5 / 8.5; M = 4 at 500 2.7 / 4.4; FP32 M = 8 at 100, 500 1.5 / 2.7,
-// 2.7 / 2.6; M = 12 at 320, 500 2.9 / 3.8, 3.9 / 3.8.
-int column_cells(bool dp, int m) { return m == 12 ? (dp ? 300 : 450) : m == 8 ? 450 : 512; }
+// per step, cluster / tiles, below and above each line: M = 12 FP64 at 272, 304 cells 7.96 / 8.29, 8.76 /
+// 8.44, FP32 at 336, 400 2.85 / 3.03, 3.15 / 3.02; M = 8 FP64 at 400, 464 5.99 / 6.32, 6.64 / 6.30, FP32
+// at 368, 432 2.32 / 2.51, 2.58 / 2.51; M = 6, 4, 3 at 512 FP64 4.41 / 5.23, 2.57 / 4.18, 1.78 / 6.14,
+// FP32 1.98 / 2.22, 1.51 / 2.04, 0.94 / 2.08.
+int column_cells(bool dp, int m) { return m == 12 ? (dp ? 288 : 368) : m == 8 ? (dp ? 432 : 400) : 512; }
 
 // The same for slices the caller chose (lbm_set_variant): the plan's shape where it has as many, else
 // 32 places in FP32, and in FP64 the fewest cells that fill a warp or two evenly (M = 8, two slices,
