@@ -205,8 +205,9 @@ lbm_status lbm_get_transport(const lbm_sim *sim, int *order);
  * lbm_warm_start) and the diagnostics stay planar on the host side; lbm_solve's refinement
  * sweeps run on the planar layout and return the state to the tiled one.
  * It changes speed, not results beyond rounding order.
- * lbm_init picks a default; lbm_set_variant returns LBM_EUNSUPPORTED for a combination
- * without a compiled kernel.  Used by the autotuner.  Call between steps only. */
+ * lbm_init picks a default, which lbm_get_variant answers until another variant is set; setting
+ * that answer leaves the choice to the library or returns it to it.  lbm_set_variant returns
+ * LBM_EUNSUPPORTED for a combination without a compiled kernel.  Used by the autotuner.  Call between steps only. */
 lbm_status lbm_set_variant(lbm_sim *sim, int warps_per_segment, int load_path);
 lbm_status lbm_get_variant(const lbm_sim *sim, int *warps_per_segment, int *load_path);
 

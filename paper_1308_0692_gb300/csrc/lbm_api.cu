@@ -59,7 +59,7 @@ struct lbm_sim {
     double dt, dx, dy, omega, u_ref;
     cudaStream_t stream;
     int lanes;            // warps per 32-cell segment of the step kernel (load paths 0, 1: velocity slices)
-    bool lanes_set;       // lanes chosen by lbm_set_variant; else tile_plan picks the slices of load path 0
+    bool lanes_set;       // a variant other than the default chosen; else tile_plan picks the slices of load path 0
     int slices;           // velocity slices of load paths 0 and 1
     bool column;          // a one-column channel whose steps run together on a cluster (step_column.cu)
     int prefetch;         // load path of the wall-free cells (lbm_set_variant)
@@ -1223,7 +1223,8 @@ lbm_status lbm_set_variant(lbm_sim *s, int warps_per_segment, int prefetch)
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(e, "changing the state layout");
     s->prefetch = prefetch;
-    s->lanes_set = true;
+    // what lbm_get_variant answers before any choice stands for the library's own
+    s->lanes_set = prefetch != 0 || warps_per_segment != default_lanes_per_cell(s->prob.prec, s->vs.m);
     return set_lanes(s, warps_per_segment);
 }
 

@@ -318,7 +318,8 @@ def lbm_set_variant(sim: Sim, warps_per_segment: int, prefetch: int = 0):
     """Step kernel: velocity slices of a cell (load paths 2 and up: warps per 32-cell segment)
     and load path (0 and 1 registers, one kernel for all cells, 2/3 TMA segments, 4 to 7 the
     column march, 8 the column march on the strip-tiled state; the C header lists which
-    combinations exist)."""
+    combinations exist).  The pair that lbm_get_variant answers before any choice stands for the
+    library's own choice by the grid."""
     _check(_load().lbm_set_variant(sim.handle, int(warps_per_segment), int(prefetch)))
 
 
