@@ -154,12 +154,16 @@ cudaError_t launch_widen(const float *src, double *dst, long count, cudaStream_t
 // Work enqueued on `waiter` from here on runs after what `first` holds now.
 inline cudaError_t stream_after(cudaStream_t waiter, cudaStream_t first)
 {
-    // the callers end with a synchronisation: a stream under capture is refused before the capture
-    // takes the other stream in
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(first, &cap);
-    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
-    if (e != cudaSuccess || waiter == first) return e;
+    // the callers end with a synchronisation: with either stream under capture they are refused before
+    // the capture takes the other one in, or an event from outside it in and is lost
+    cudaError_t e = cudaSuccess;
+    for (cudaStream_t s : {first, waiter}) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        e = cudaStreamIsCapturing(s, &cap);
+        if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+        if (e != cudaSuccess) return e;
+    }
+    if (waiter == first) return e;
     cudaEvent_t ev;
     e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e != cudaSuccess) return e;
