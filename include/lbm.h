@@ -385,7 +385,7 @@ lbm_status lbm_batch_set_state(lbm_batch *b, int i, const double *h);
 typedef struct lbm_mlp lbm_mlp;
 lbm_status lbm_batch_warm_start(lbm_batch *b, int i, lbm_mlp *mlp, double kn, double u_w);
 /* Moments of instance i (as lbm_moments) into device FP64 [6][ny][nx]: rho, ux, uy, pxx,
- * pxy, pyy.  Stream-ordered. */
+ * pxy, pyy.  Stream-ordered; refused (LBM_ECUDA) while the batch's stream is captured. */
 lbm_status lbm_batch_moments(lbm_batch *b, int i, double *out_dev);
 /* Mixed-precision refinement of every instance, all instances at once (the batched form of
  * lbm_solve's refinement sweeps; not in the paper).  Each sweep evaluates the defect

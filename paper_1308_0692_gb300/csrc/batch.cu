@@ -2370,6 +2370,11 @@ lbm_status lbm_batch_moments(lbm_batch *b, int i, double *out_dev)
 {
     if (!b || !out_dev) return bfail(LBM_EINVAL, "NULL argument");
     if (i < 0 || i >= (int)b->inst.size()) return bfail(LBM_EINVAL, "instance index out of range");
+    // the launch carries the step that the batch stands at: a graph would replay it at later ones
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(b->stream, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+    if (e != cudaSuccess) return bfail(LBM_ECUDA, std::string("instance moments: ") + cudaGetErrorString(e));
     const BatchArgs a = make_args(b, 1, 0.0);
     const BatchInst &I = b->inst[i];
     const long blocks = I.tiled ? (long)((I.nx + 31) / 32) * I.ny : (I.ncells + 31) / 32;
@@ -2378,7 +2383,7 @@ lbm_status lbm_batch_moments(lbm_batch *b, int i, double *out_dev)
         inst_moments_kernel<8><<<(unsigned)blocks, 256, 0, b->stream>>>(b0, b1, b->d_frozen + i, b->step, I, a, 1.0 / I.inv_u_ref, out_dev);
     else
         inst_moments_kernel<4><<<(unsigned)blocks, 192, 0, b->stream>>>(b0, b1, b->d_frozen + i, b->step, I, a, 1.0 / I.inv_u_ref, out_dev);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     return e == cudaSuccess ? LBM_OK : bfail(LBM_ECUDA, std::string("instance moments: ") + cudaGetErrorString(e));
 }
 

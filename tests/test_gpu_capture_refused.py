@@ -45,3 +45,16 @@ def test_warm_start_with_either_stream_under_capture(kind, captured):
     _refused_under_capture(stream if captured == "object" else net_stream, call)
     call()
     assert np.array_equal(state(), h)
+
+
+def test_batch_moments_under_capture():
+    stream = torch.cuda.Stream()
+    b = lbm.lbm_batch_init(lbm.lbm_make_velocity_set(lbm.LBM_HALF_RANGE_GH, 4), [_problem()], stream=stream)
+    lbm.lbm_batch_advance(b, 3, 0.0)
+    out = torch.full((6, 32, 32), -7.0, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    _refused_under_capture(stream, lambda: lbm.lbm_batch_moments(b, 0, out.data_ptr()))
+    assert bool((out == -7.0).all())
+    lbm.lbm_batch_moments(b, 0, out.data_ptr())
+    stream.synchronize()
+    assert bool((out[0] > 0.5).all())
