@@ -3,9 +3,14 @@
 // mlp_grad_kernel: dW_l = g_l^T a_l for the four layers in one launch, K = the batch rows
 // (128-row tiles padded with zero gradients).  A CTA takes one 128 x 128 tile (128 x 16 for the
 // 4-wide input layer) of one layer and one of the K-splits: a TMA producer, one thread issuing
-// tcgen05.mma, a ring of four stages, the accumulator in tensor memory -- and stores its partial
+// tcgen05.mma, a ring of four stages, the accumulators in tensor memory -- and stores its partial
 // tile column by column (lane = row: contiguous).  Twelve tiles times at most twelve splits are
-// 144 CTAs, one wave of the 152 SMs.
+// 144 CTAs, one wave of the 152 SMs.  The CTA's steps go to four accumulators, a quarter of them
+// each: FP32 additions in tensor memory lose half an ulp on average, so the error grows with the
+// length of a chain, and 48 chains are shorter than twelve (128 rows over and over, 8192 and 32768 in
+// all: relative error of the gradients 1.2e-7 and 6.1e-7; with one accumulator 6.2e-7 and 2.8e-6).
+// They fill the tensor memory; no other kernel of the network fits on the SM beside this one's
+// shared memory.
 //
 // mlp_reduce_adam_kernel: adds the splits in ascending order, turns the 32 x 32 block through
 // shared memory, applies Adam on the FP32 master weights and refreshes both BF16 copies
@@ -25,6 +30,7 @@ namespace {
 constexpr int STAGES = 4;
 constexpr int STAGE = 2 * UM * 128;                 // bytes: A and B tiles of one K step
 constexpr int SMEM = STAGES * STAGE + 1024;
+constexpr int ACCS = 4, ACC = 128;                  // accumulators of a CTA, 128 columns each
 
 // tile t of the list: layer, first row (of N_l), first column (of K_l), columns
 struct Tile {
@@ -56,6 +62,7 @@ __global__ void __launch_bounds__(256, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const Tile t = tile_of(blockIdx.x);
     const int kt0 = blockIdx.y * kper, kt1 = min(ktiles, kt0 + kper);
+    const int chain = max(1, (kt1 - kt0 + ACCS - 1) / ACCS);      // steps of an accumulator
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -65,7 +72,7 @@ __global__ void __launch_bounds__(256, 1)
         bar_init(&accf, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (warp == 0) tmem_alloc(&s_tmem, 128);
+    if (warp == 0) tmem_alloc(&s_tmem, ACCS * ACC);
     asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;\n" ::: "memory");
     fence_before_sync();
     __syncthreads();
@@ -104,7 +111,7 @@ __global__ void __launch_bounds__(256, 1)
             const uint64_t da = smem_desc(st), db = smem_desc(st + UM * 128);
 #pragma unroll
             for (int k = 0; k < UK / 16; ++k)   // advance 16 BF16 = 32 bytes along K inside the swizzle row
-                mma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (done | k) ? 1u : 0u);
+                mma_bf16(tmem + (uint32_t)(done / chain * ACC), da + 2 * k, db + 2 * k, idesc, (done % chain | k) ? 1u : 0u);
             mma_commit(&empty[s]);
         }
         mma_commit(&accf);
@@ -115,21 +122,28 @@ __global__ void __launch_bounds__(256, 1)
     fence_after_sync();
     // ---- epilogue: warp w takes rows 32 (w % 4).., columns 64 (w / 4)..; column-major partial tile
     float *out = part + ((long)blockIdx.x * gridDim.y + blockIdx.y) * (128 * 128) + (warp & 3) * 32 + lane;
-    const bool any = kt1 > kt0;
+    const int accs = kt1 > kt0 ? (kt1 - kt0 + chain - 1) / chain : 0;
     __syncwarp();
 #pragma unroll 1
     for (int c0 = (warp >> 2) * 64; c0 < (warp >> 2) * 64 + 64 && c0 < t.n; c0 += 32) {
         float v[32];
-        tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, v);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = 0.f;
+        for (int q = 0; q < accs; ++q) {
+            float u[32];
+            tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(q * ACC + c0), u);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] += u[j];
+        }
 #pragma unroll
         for (int j = 0; j < 32; ++j)
-            if (c0 + j < t.n) out[(c0 + j) * 128] = any ? v[j] : 0.f;
+            if (c0 + j < t.n) out[(c0 + j) * 128] = v[j];
     }
     fence_before_sync();
     __syncthreads();
     if (warp == 0) {
         fence_after_sync();
-        tmem_free(tmem, 128);
+        tmem_free(tmem, ACCS * ACC);
     }
 }
 
