@@ -138,6 +138,8 @@ bool kernel_m_supported(int m) { return m == 3 || m == 4 || m == 6 || m == 8 || 
 bool march_grid_ok(const lbm_problem *p) { return p->nx % 64 == 0 && p->nx >= 128 && p->ny >= 10; }
 bool tile_eligible(const lbm_problem *p) { return p->prec == LBM_FP32_PERTURB && p->geom == LBM_CAVITY && march_grid_ok(p); }
 
+long most_tile_blocks(int prec, int m, int nx, int ny);
+
 struct Layout {
     size_t off_buf[4];
     size_t off_tab64, off_tab32, off_hdr, off_partials, off_result, off_moments, off_fy, off_fx, off_wsegs;
@@ -172,9 +174,9 @@ Layout make_layout(const lbm_vset *vs, const lbm_problem *p)
     L.wall_cap = 2 * (p->nx + p->ny) + 4;
     L.off_wsegs = off;
     off = align256(off + sizeof(int) * L.wall_cap);
-    // the finest launch has four cells a block (tile_plan) or, on the segment paths, 32-cell
-    // segments and the wall kernel's blocks; norms use at most 152*8 blocks
-    long nb = std::max((ncells + 3) / 4 + 8L * p->nx, (ncells + 31) / 32 + L.wall_cap);
+    // the blocks of the finest launch that a variant or the refinement makes: blocks of step_tile.cuh,
+    // or on the segment paths 32-cell segments and the wall kernel's; norms use at most 152*8 blocks
+    long nb = std::max(most_tile_blocks(p->prec, vs->m, p->nx, p->ny), (ncells + 31) / 32 + L.wall_cap);
     if (nb < 152 * 8) nb = 152 * 8;
     L.npartials = (int)nb;
     L.off_partials = off;
@@ -469,6 +471,21 @@ TilePlan tile_plan_for(bool dp, int m, long ncells, int ns)
     if (!dp) return {ns, 32, ns == 1 ? 2 : 1};
     if (ns == 6) return {6, 16, 1};
     return {ns, 8, ns == 1 || ns == 3 ? 4 : ns == 2 ? 2 : 1};
+}
+
+// Most blocks of step_tile.cuh in a launch on this grid: the plan's, those of every choice of slices,
+// and for FP32 the refinement's defect (FP64) and correction passes.
+long most_tile_blocks(int prec, int m, int nx, int ny)
+{
+    const bool dp = prec == LBM_FP64;
+    const long ncells = (long)nx * ny;
+    long most = 0;
+    auto take = [&](const TilePlan &t) { most = std::max(most, tile_blocks(nx, ny, t.w, t.r)); };
+    take(tile_plan(dp, m, ncells));
+    if (!dp) take(tile_plan(true, m, ncells));
+    for (int ns = 1; ns <= m; ++ns)
+        if (step_supported(prec, m, ns, 0) || step_supported(prec, m, ns, 1)) take(tile_plan_for(dp, m, ncells, ns));
+    return most;
 }
 
 int grid_for(long ncells, int lanes)
