@@ -711,12 +711,23 @@ __host__ __device__ constexpr int half_warps(int n) { return (2 * n) % 4 == 0 ? 
 // 129.2 and 23.9 / 22.0; 200^2 N = 6, 8 cells 79.3 / 76.8 and 27.9 / 24.9, N = 3 FP32 13.3 / 10.1;
 // one in three or four the same but 512^2 FP32 (23.8).  A grid that is in flight almost at once
 // starts its longest chains first: 128^2 N = 4, 4 cells FP64 27.4 / 28.3.
+//
+// The next step's blocks are set up while this one runs.  With interface cells that begins with the
+// block, as their projection matrices take time.  Without, it begins when a block has stored: blocks
+// that wait among running ones leave some SMs two blocks of the next step and others none.  us a step,
+// not set up ahead / at the start / at the end (the kernel before this form): FP64 full-range only
+// 128^2 N = 4 14.7 / 21.3 / 11.9 (16.7), N = 2 7.5 / 10.9 / 5.3 (8.5), 192^2 N = 2 9.9 / 14.1 / 7.3
+// (10.5); half-range only 64^2 N = 4 14.6 / 23.3 / 12.2 (18.7), N = 3 14.7 / 22.5 / 13.2 (20.8); FP32
+// N = 3 192^2 6.4 / 9.1 / 4.6 (6.4), 144^2 half-range N = 2 10.5 / 12.2 / 8.1 (10.6).  From two and a
+// half blocks an SM on, FP64 with more than 16 velocities gains nothing by it (512 blocks, N = 6
+// half-range 61.2 / 57.0 / 59.1; 392, N = 3 16.7 / 14.1 / 14.5).
 struct StepLists {
     const int *cells;          // interface cells
     int ncells;
     const int2 *tiles[2];      // half-range, full-range tiles with a plain cell
     int ntiles[2];
     int every;                 // one block in `every` takes interface cells, until they are dealt (1 or 2)
+    int early;                 // a block lets the next step's blocks be set up when it starts, else when it ends
 };
 
 // blocks a SM the FP32 build asks for: eight (64 registers a thread) where that does not
@@ -741,7 +752,7 @@ __global__ void __launch_bounds__(32 * HWARPS, hybrid_min_blocks<N, TS>()) hybri
     const int hbk = (L.ntiles[0] + HWARPS / GH - 1) / (HWARPS / GH);
     // the next step's blocks are set up while this one runs (for the interface cells with the
     // projection matrices in shared memory) and wait for it before they read the state
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (L.early) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const bool interface = bid < ifb * L.every && bid % L.every == 0;
     // block among the interface blocks, or among the others
     const int k0 = interface ? bid / L.every : bid - min(ifb, bid / L.every + 1);
@@ -762,11 +773,12 @@ __global__ void __launch_bounds__(32 * HWARPS, hybrid_min_blocks<N, TS>()) hybri
     } else {
         plain_tiles<N, 1>(pf, L.tiles[1], L.ntiles[1], k0 - hbk, resid, u.fx);
     }
+    if (!L.early) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
 template <int N, typename TS>
 cudaError_t launch_step_n(const HybArgs &a, const PlainArgs<TS> &ph, const PlainArgs<TS> &pf, const StepLists &L,
-                          int resid, cudaStream_t st)
+                          int resid, int sms, cudaStream_t st)
 {
     constexpr int GH = half_warps(N);
     const int ifb = (L.ncells + HWARPS - 1) / HWARPS;
@@ -774,7 +786,8 @@ cudaError_t launch_step_n(const HybArgs &a, const PlainArgs<TS> &ph, const Plain
     const int blocks = ifb + others;
     if (blocks == 0) return cudaSuccess;
     StepLists D = L;
-    D.every = blocks >= 4 * 152 && others >= ifb ? 2 : 1;
+    D.every = blocks >= 4 * sms && others >= ifb ? 2 : 1;
+    D.early = ifb > 0 || (sizeof(TS) == 8 && N > 2 && 2 * blocks >= 5 * sms);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(32 * HWARPS);
@@ -789,14 +802,14 @@ cudaError_t launch_step_n(const HybArgs &a, const PlainArgs<TS> &ph, const Plain
 
 template <typename TS>
 cudaError_t launch_hybrid_step(int n, const HybArgs &a, const PlainArgs<TS> &ph, const PlainArgs<TS> &pf,
-                               const StepLists &L, int resid, cudaStream_t st)
+                               const StepLists &L, int resid, int sms, cudaStream_t st)
 {
     switch (n) {
-    case 2: return launch_step_n<2, TS>(a, ph, pf, L, resid, st);
-    case 3: return launch_step_n<3, TS>(a, ph, pf, L, resid, st);
-    case 4: return launch_step_n<4, TS>(a, ph, pf, L, resid, st);
-    case 5: return launch_step_n<5, TS>(a, ph, pf, L, resid, st);
-    case 6: return launch_step_n<6, TS>(a, ph, pf, L, resid, st);
+    case 2: return launch_step_n<2, TS>(a, ph, pf, L, resid, sms, st);
+    case 3: return launch_step_n<3, TS>(a, ph, pf, L, resid, sms, st);
+    case 4: return launch_step_n<4, TS>(a, ph, pf, L, resid, sms, st);
+    case 5: return launch_step_n<5, TS>(a, ph, pf, L, resid, sms, st);
+    case 6: return launch_step_n<6, TS>(a, ph, pf, L, resid, sms, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -986,6 +999,7 @@ struct lbm_hybrid {
     long unknowns;           // values of the packed state
     long tiled;              // doubles of the tiled device state (tiles padded to 32 cells)
     cudaStream_t stream;
+    int sms;                 // of the device
     HybTabT<double> *d_tab;  // the tables for the FP64 kernels
     HybTabT<float> *d_tab32; // and for the FP32 march
     int *d_poff, *d_toff;    // packed offsets; tiled offsets of velocity 0 of each cell
@@ -1132,7 +1146,7 @@ cudaError_t hybrid_launch(const lbm_hybrid *hb, const HybArgs &a0, int resid)
         L.ntiles[t] = hb->n_tiles[t];
     }
     return launch_hybrid_step<TS>(hb->n_half, a, plain_args<TS>(hb, 0, a), plain_args<TS>(hb, 1, a), L, resid,
-                                  hb->stream);
+                                  hb->sms, hb->stream);
 }
 
 // the two-stage reduction of the residual partials into d_res[0..1]
@@ -1179,6 +1193,7 @@ lbm_status lbm_hybrid_init(int geom, int n_half, int nx, int ny, double kn, doub
     hb->u_top = u_top;
     hb->cfl = cfl;
     hb->stream = (cudaStream_t)stream;
+    hb->sms = 0;
     hb->cur = 0;
     hb->have_resid = false;
     hb->d_tab = nullptr;
@@ -1379,7 +1394,10 @@ lbm_status lbm_hybrid_init(int geom, int n_half, int nx, int ny, double kn, doub
                 }
             }
         }
-    cudaError_t e = cudaMalloc(&hb->d_tab, sizeof(HybTabT<double>));
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&hb->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaMalloc(&hb->d_tab, sizeof(HybTabT<double>));
     if (e == cudaSuccess) e = cudaMalloc(&hb->d_tab32, sizeof(HybTabT<float>));
     if (e == cudaSuccess) e = cudaMalloc(&hb->d_poff, sizeof(int) * (nc + 1));
     if (e == cudaSuccess) e = cudaMalloc(&hb->d_toff, sizeof(int) * nc);
