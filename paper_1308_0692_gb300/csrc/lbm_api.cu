@@ -398,6 +398,12 @@ void fill_args(lbm_sim *s, const TableHeader &hdr)
             a.so_c_f[ax][i] = (float)a.so_c[ax][i];
         }
     }
+    for (int i = 0; i < v.m / 2; ++i) {
+        a.xi_p[i] = make_float2(a.xi_f[2 * i], a.xi_f[2 * i + 1]);
+        a.nux_p[i] = make_float2(a.nux_f[2 * i], a.nux_f[2 * i + 1]);
+        a.nuy_p[i] = make_float2(a.nuy_f[2 * i], a.nuy_f[2 * i + 1]);
+        a.w1_p[i] = make_float2(a.w1_f[2 * i], a.w1_f[2 * i + 1]);
+    }
     a.omega = s->omega;
     a.b = 1.0 - s->omega;
     scale_tables(a, v.m);

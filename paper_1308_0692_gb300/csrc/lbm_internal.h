@@ -96,6 +96,9 @@ struct StepArgs {
     double inv_dy_wall;     // 1 / sum_{xi_y>0} xi_y w  (bottom / top walls)
     double u_bottom, u_top; // wall speeds
     double inv_u_ref;       // 1 / u_ref
+    // nodes (2 i, 2 i + 1) of xi_f, nux_f, nuy_f, w1_f as pairs, for the kernels that gain by loading two
+    // coefficients at once (xi_f itself lies 4 bytes off an 8-byte boundary): step_tma.cuh, step_march.cuh
+    float2 xi_p[LBM_MAX_M / 2], nux_p[LBM_MAX_M / 2], nuy_p[LBM_MAX_M / 2], w1_p[LBM_MAX_M / 2];
 };
 
 // Blocks of step_tile.cuh over an nx x ny grid with W places of R rows a block.

@@ -133,6 +133,11 @@ step_march_kernel(const StepArgs a)
 
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    // coefficients in pairs (StepArgs): M = 8 on the planar state with five slots 361 us a step at 2048^2
+    // against 371; the other forms lose by it (M = 12 planar 902 to 918, tiled the same)
+    constexpr bool PAIRS = M == 8 && S == 5 && TILED == 0 && RPL == 2;
+    auto of_x = [&](const float2 *p, const float *t, int ix) { return PAIRS ? (ix % 2 ? p[ix / 2].y : p[ix / 2].x) : t[ix]; };
+    auto of_row = [&](const float2 *p, const float *t, int r) { return PAIRS ? (r ? p[g].y : p[g].x) : t[g * RPL + r]; };
     const long ncells = a.ncells;
     const int nx = a.nx;
     const int nstrips = a.march_strips, nchunks = a.march_chunks;
@@ -188,7 +193,7 @@ step_march_kernel(const StepArgs a)
         if constexpr (ORDER == 2) {
             v = (float)(1.0 - a.so_p[0][ix] - a.so_p[1][g * RPL + r]);
         } else {
-            v = 1.f - a.nux_f[ix] - a.nuy_f[g * RPL + r];
+            v = 1.f - of_x(a.nux_p, a.nux_f, ix) - of_row(a.nuy_p, a.nuy_f, r);
         }
         a0r[k] = make_float2(v, v);
     }
@@ -208,9 +213,9 @@ step_march_kernel(const StepArgs a)
     }
 #pragma unroll
     for (int ix = 0; ix < M; ++ix) {
-        nux2[ix] = make_float2(a.nux_f[ix], a.nux_f[ix]);
-        xi2[ix] = make_float2(a.xi_f[ix], a.xi_f[ix]);
-        w2[ix] = make_float2(a.w1_f[ix], a.w1_f[ix]);
+        nux2[ix] = make_float2(of_x(a.nux_p, a.nux_f, ix), of_x(a.nux_p, a.nux_f, ix));
+        xi2[ix] = make_float2(of_x(a.xi_p, a.xi_f, ix), of_x(a.xi_p, a.xi_f, ix));
+        w2[ix] = make_float2(of_x(a.w1_p, a.w1_f, ix), of_x(a.w1_p, a.w1_f, ix));
     }
     // plane offset of this lane's copy (lanes < NV issue one line each per row)
     const int kc = lane < NV ? lane : 0;
@@ -332,8 +337,8 @@ step_march_kernel(const StepArgs a)
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
             const int iy = g * RPL + r;
-            const float wom = om * a.w1_f[iy];
-            const float xiy = a.xi_f[iy];
+            const float wom = om * of_row(a.w1_p, a.w1_f, r);
+            const float xiy = of_row(a.xi_p, a.xi_f, r);
             const float2 q2 = __fmul2_rn(make_float2(wom, wom), __ffma2_rn(make_float2(xiy, xiy), y2, r2));
             const float2 jj2 = __fmul2_rn(make_float2(wom, wom), x2);
             float *rowp = hn + (long)(iy * M) * ncells + cell;
@@ -374,7 +379,7 @@ step_march_kernel(const StepArgs a)
 #pragma unroll
             for (int r = 0; r < RPL; ++r) {
                 const int iy = g * RPL + r;
-                const float nuy = a.nuy_f[iy];
+                const float nuy = of_row(a.nuy_p, a.nuy_f, r);
                 const float2 nuy2 = make_float2(nuy, nuy);
                 // row sums in NACC independent partial sums (short dependency chains)
                 constexpr int NACC = 4;
@@ -436,7 +441,7 @@ step_march_kernel(const StepArgs a)
                 }
                 const float2 R = __fadd2_rn(__fadd2_rn(R2[0], R2[1]), __fadd2_rn(R2[2], R2[3]));
                 const float2 X = __fadd2_rn(__fadd2_rn(X2[0], X2[1]), __fadd2_rn(X2[2], X2[3]));
-                const float xiy = a.xi_f[iy];
+                const float xiy = of_row(a.xi_p, a.xi_f, r);
                 rho2 = __fadd2_rn(rho2, R);
                 jx2 = __fadd2_rn(jx2, X);
                 jy2 = __ffma2_rn(make_float2(xiy, xiy), R, jy2);
@@ -500,8 +505,8 @@ step_march_kernel(const StepArgs a)
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
             const int iy = g * RPL + r;
-            const float wom = om * a.w1_f[iy];
-            const float xiy = a.xi_f[iy];
+            const float wom = om * of_row(a.w1_p, a.w1_f, r);
+            const float xiy = of_row(a.xi_p, a.xi_f, r);
             const float2 q2 = __fmul2_rn(make_float2(wom, wom), __ffma2_rn(make_float2(xiy, xiy), jy2, rho2));
             const float2 jj2 = __fmul2_rn(make_float2(wom, wom), jx2);
             float *rowp = TILED ? hn + tcell + (long)(iy * M) * LBM_TILE_W : hn + (long)(iy * M) * ncells + cell;

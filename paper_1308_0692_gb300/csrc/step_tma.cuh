@@ -82,7 +82,11 @@ struct TmaShape {
     static constexpr int SMEM = Shape<G>::WARPS * BYTES_PER_WARP + Shape<G>::WARPS * 8 + 16;
 };
 
-template <int M, int G, bool RESID>
+// PAIRS: the coefficients of a velocity pair in one load.  Without, the kernel that takes only these
+// segments is 2 % slower (2048^2, M = 8, four warps 529 us a step against 538, M = 12 with four and three
+// 1502 / 1519 and 1511 / 1539).  The merged one keeps single loads: M = 8 530, with tables at 8-byte
+// boundaries 540 (M = 12, four warps, 1478 and 1464).
+template <int M, int G, bool RESID, bool PAIRS>
 __device__ __forceinline__ void tma_body(const StepArgs &a, const int bid)
 {
     using TC = float;
@@ -152,6 +156,7 @@ __device__ __forceinline__ void tma_body(const StepArgs &a, const int bid)
     // issue-bound kernel.  Transport in the form (1 - nu_x - nu_y) h + nu_x h_x + nu_y h_y.
     // A pair never straddles the sign change of xi_x (M/2 is even for M = 8, 12).
     static_assert((M / 2) % 2 == 0, "velocity pairs must not straddle xi_x = 0");
+    auto pair = [](const float2 *p, const float *t, int ix) { return PAIRS ? p[ix / 2] : make_float2(t[ix], t[ix + 1]); };
     float2 hs[RPL * M / 2];
     TC rho = 0, jx = 0, jy = 0;
     if (compute) {
@@ -170,14 +175,14 @@ __device__ __forceinline__ void tma_body(const StepArgs &a, const int bid)
                 const float2 hc = make_float2(cen[k * CEN + 4 + lane], cen[(k + 1) * CEN + 4 + lane]);
                 const float2 hx = make_float2(cen[k * CEN + sx + lane], cen[(k + 1) * CEN + sx + lane]);
                 const float2 hy = make_float2(yn[k * YN + lane], yn[(k + 1) * YN + lane]);
-                const float2 nux = make_float2(a.nux_f[ix], a.nux_f[ix + 1]);
-                const float2 a0 = make_float2(1.f - a.nux_f[ix] - nuy, 1.f - a.nux_f[ix + 1] - nuy);
+                const float2 nux = pair(a.nux_p, a.nux_f, ix);
+                const float2 a0 = make_float2(1.f - nux.x - nuy, 1.f - nux.y - nuy);
                 float2 v = __fmul2_rn(a0, hc);
                 v = __ffma2_rn(nux, hx, v);
                 v = __ffma2_rn(nuy2, hy, v);
                 hs[r * (M / 2) + pp] = v;
                 R2 = __fadd2_rn(R2, v);
-                X2 = __ffma2_rn(make_float2(a.xi_f[ix], a.xi_f[ix + 1]), v, X2);
+                X2 = __ffma2_rn(pair(a.xi_p, a.xi_f, ix), v, X2);
             }
             const TC R = R2.x + R2.y, X = X2.x + X2.y;
             rho += R;
@@ -218,8 +223,8 @@ __device__ __forceinline__ void tma_body(const StepArgs &a, const int bid)
             for (int pp = 0; pp < M / 2; ++pp) {
                 const int ix = 2 * pp;
                 const int k = r * M + ix;
-                const float2 t = __ffma2_rn(make_float2(a.xi_f[ix], a.xi_f[ix + 1]), jj2, q2);
-                const float2 v = __ffma2_rn(make_float2(a.w1_f[ix], a.w1_f[ix + 1]), t,
+                const float2 t = __ffma2_rn(pair(a.xi_p, a.xi_f, ix), jj2, q2);
+                const float2 v = __ffma2_rn(pair(a.w1_p, a.w1_f, ix), t,
                                             __fmul2_rn(b2, hs[r * (M / 2) + pp]));
                 if (RESID) {
                     const float2 hc = make_float2(cen[k * CEN + 4 + lane], cen[(k + 1) * CEN + 4 + lane]);
@@ -264,7 +269,7 @@ __device__ __forceinline__ void tma_body(const StepArgs &a, const int bid)
 template <int M, int G, bool RESID>
 __global__ void __launch_bounds__(Shape<G>::THREADS) step_tma_kernel(const StepArgs a)
 {
-    tma_body<M, G, RESID>(a, blockIdx.x);
+    tma_body<M, G, RESID, true>(a, blockIdx.x);
 }
 
 // One launch for the whole step: the wall segments first (blocks [0, wall_blocks), the
@@ -276,7 +281,7 @@ __global__ void __launch_bounds__(Shape<G>::THREADS) step_tma_merged_kernel(cons
     if ((int)blockIdx.x < a.wall_blocks)
         wall_body<M, G, RESID, false>(a, blockIdx.x);
     else
-        tma_body<M, G, RESID>(a, blockIdx.x - a.wall_blocks);
+        tma_body<M, G, RESID, false>(a, blockIdx.x - a.wall_blocks);
 }
 
 // Opt the kernels into their dynamic shared memory (once per process, before any launch
