@@ -8,7 +8,7 @@ ghosts, moments, relaxation; the residual reduction on every 10th step).
 
 Metric: node-velocity updates per second (cells x velocities x steps / s).
 
-  python bench.py [--gpus N] [--steps K] [--warmup W] [--impl own|reference]
+  python bench.py [--gpus N] [--steps K] [--warmup W] [--impl own|reference] [--record FILE]
 
 With --gpus N > 1 (launched by torchrun) every rank marches its own replica of the
 workload (the single-domain march has no data-parallel split without a halo exchange,
@@ -682,7 +682,7 @@ def run_time_to_residual(dist):
 
 def ttr_summary(ttr: dict, oracle_rate: float | None) -> dict:
     """A short digest of the time-to-residual runs (seconds, speed-ups, worst velocity error
-    against the FP64 march, instance counts), printed as the line's last key."""
+    against the FP64 march, instance counts), the line's last key."""
     def r3(x):
         return None if x is None else float(f"{x:.4g}")
     full, sub = ttr["held_out_256"], ttr["ablation_32"]
@@ -844,6 +844,46 @@ def run_reference(args, dist: Dist):
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
 
 
+# ---------------------------------------------------------------- the printed line
+def bench_line(out: dict) -> dict:
+    """What is printed of a run's record: the headline, the end-to-end figure, clocks and roofline
+    whole, of the rest the figures alone.  A log that keeps the last 3,000 characters keeps all of it;
+    --record writes the whole record (every call's parts, the autotuner's times, steps and errors of
+    each instance)."""
+    def r4(x):
+        return None if x is None else float(f"{x:.4g}")
+
+    def pick(d, *keys):
+        return {k: r4(d[k]) if isinstance(d[k], float) else d[k] for k in keys if k in d}
+
+    line = {k: v for k, v in out.items() if not isinstance(v, (dict, list)) or k in ("clocks", "last_residual", "ttr_summary")}
+    c = out["config"]
+    line["config"] = {k: c[k] for k in c if k not in ("variant", "cold_start")}
+    line["config"]["variant"] = "{warps_per_segment} warps, {load_path}".format(**c["variant"])
+    line["roofline"] = pick(out["roofline"], "bound", "achieved", "peak", "unit", "frac", "peak_source", "avg_launch_ms",
+                            "algorithmic_bytes_per_launch", "traffic")
+    if "e2e" in out:
+        e = out["e2e"]
+        line["e2e"] = {k: e[k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_call") if k in e}
+        line["e2e"]["call"] = "lbm_set_state_f32(pinned host) + lbm_step(100) + lbm_residual + lbm_moments(ux, uy)"
+        if "fp64_host_upload" in e:
+            line["e2e"]["fp64_host_upload"] = r4(e["fp64_host_upload"]["value"])
+    if "fp64" in out:
+        line["fp64"] = dict(pick(out["fp64"], "value", "ms_per_step"), pipe_frac=r4(out["fp64"]["fp64_pipe"]["frac"]))
+    if "second_order" in out:
+        so = out["second_order"]
+        line["second_order"] = {"fp32": dict(pick(so["fp32"], "value", "ms_per_step"), frac=r4(so["fp32"]["roofline"]["frac"])),
+                                "fp64": pick(so["fp64"], "value", "ms_per_step")}
+    if "cpu_baseline" in out:
+        line["cpu_baseline"] = pick(out["cpu_baseline"], "value", "unit", "cores", "kind", "single_thread_value")
+    if "configs_time_to_residual" in out:         # case: seconds of the oracle, the FP64 and the refined FP32 march
+        line["configs_s"] = {c["case"]: [r4(c[k]["seconds"]) for k in ("oracle", "gpu_fp64", "gpu_fp32_dc")]
+                             for c in out["configs_time_to_residual"]}
+    if "ttr_summary" in line:
+        line["ttr_summary"] = line.pop("ttr_summary")
+    return line
+
+
 # ---------------------------------------------------------------- main
 def main(argv=None):
     ap = argparse.ArgumentParser()
@@ -861,6 +901,7 @@ def main(argv=None):
                     help="2: time the second-order variant of the workload instead (profiling)")
     ap.add_argument("--fp64-only", action="store_true",
                     help="time only the plain FP64 march of the workload (profiling of the FP64 step)")
+    ap.add_argument("--record", default=None, help="file for the whole record, of which the printed line is a digest")
     args = ap.parse_args(argv)
     if args.nx:
         WORKLOAD["nx"] = WORKLOAD["ny"] = args.nx
@@ -916,7 +957,11 @@ def main(argv=None):
                              "on the 128^2 D2Q^h_64 cavity configurations",
                     "vs_warm_dc": (upd / rate) / full["warm_dc"]["seconds"] if full.get("warm_dc") else None}
             out["ttr_summary"] = ttr_summary(ttr, rate)
-        print(json.dumps(out), flush=True)
+        if args.record:
+            with open(args.record, "w") as f:
+                json.dump(out, f)
+                f.write("\n")
+        print(json.dumps(bench_line(out)), flush=True)
     dist.close()
     return 0
 
