@@ -417,26 +417,26 @@ void fill_args(lbm_sim *s, const TableHeader &hdr)
 }
 
 // Velocity slices and cells of a block of step_tile.cuh (load paths 0 and 1, the correction
-// march; dp: FP64 arithmetic, the FP64 march and the defect pass).  Measured over 19 grids
-// (1 x 100 to 512 x 512, M = 3 to 12; us per step, replayed graphs; both sides with the build
-// that the line was drawn with, the kernel has since gained 5 to 10 %: now M = 8 FP64 128^2 23.6,
-// 192^2 44.4, FP32 128^2 3.9, 333 x 251 10.1, M = 12 FP64 300^2 205, 512^2 556):
+// march; dp: FP64 arithmetic, the FP64 march and the defect pass).  Lines from 19 grids (1 x 100 to
+// 512 x 512, M = 3 to 12) and the larger ones below; us per step, replayed graphs, both sides in one
+// build:
 //   FP64 is bound by the FP64 pipe of each SM quarter, so small blocks that spread evenly win,
 //     with one velocity row a thread while the grid leaves the quarters short of warps (M = 8:
-//     64^2 12.1 against 15.6 with two rows, 128^2 25.2 against 28.1) and two or three rows a
-//     thread beyond (M = 8: 192^2 48.1 against 50.0; M = 12: 128^2 51.9 against 54.4, 300^2
-//     223.5 against 225.2, 512^2 614 against 624);
+//     64^2 12.5 against 18.1 with two rows, 128^2 23.9 against 26.9) and two or three rows a
+//     thread beyond (M = 8: 192^2 45.2 against 46.8; M = 12: one row 128^2 45.5 against 51.4, 300^2
+//     205 against 209, three rows 512^2 563 against 575);
 //   FP32 is bound by the L2's latency and traffic: 16 places with two rows a thread (M = 8:
-//     128^2 4.8; 32 places 5.9, one row a thread 6.0), 32 places where there are enough of
+//     128^2 4.1; 32 places 4.9, one row a thread 5.1), 32 places where there are enough of
 //     them to fill the chip (333 x 251 10.4 against 10.8), few cells with one row a thread
-//     (40 x 33 2.9 against 3.2); small sets whole rows a thread (M = 4: 128^2 2.7 against 2.9).
+//     (40 x 33 2.9 against 3.1); small sets whole rows a thread (M = 4: 128^2 3.0 against 3.4).
 // Beyond the L2 (two states of more than 129 MB together) narrow blocks fetch lines they use half of
-// and find fewer of the y neighbours in the L1: 32 places, and from 2M cells on two rows of cells, at 1000 x
-// 900 and 2047 x 1500 M = 12 FP32 384 to 241 and 1797 to 861 (six slices of 16 places; 331 to 336 and
-// 650 to 580 from four of 32 to two of 32 x 2 at 1.2M and 2.1M cells), M = 8 395 to 339 at 2047 x 1500,
-// M = 3 29.1 to 15.2 and 98.0 to 51.9.  FP64 with small sets takes whole rows a thread once the quarters
-// have warps enough: M = 4 at 200^2, 300 x 250, 600^2 16.5 / 24.1, 27.4 / 26.3, 118 / 98 (four slices /
-// one), M = 6 at 300 x 250, 400 x 300, 600^2 51.5 / 51.8, 79.2 / 77.8, 224 / 209 (six / two).
+// and find fewer of the y neighbours in the L1: 32 places, and from 2M cells on two rows of cells.  M = 12
+// FP32, six slices of 16 places / four of 32 / two of 32 x 2: 1000 x 900 385 / 247 / 263, 1200 x 1000 - /
+// 327 / 339, 1500 x 1400 - / 654 / 594, 2047 x 1500 1804 / 936 / 867; 2047 x 1500, one and two rows, M = 8
+// 401 / 349, M = 6 196 / 190, M = 3 with 16 and 32 places 98.2 / 52.0.  FP64 with small sets takes whole
+// rows a thread once the quarters have warps enough: M = 4 at 200^2, 300 x 250, 600^2 16.8 / 24.6, 27.7 /
+// 26.5, 119 / 98 (four slices / one), M = 6 at 300 x 250, 400 x 300, 600^2 51.9 / 52.3, 79.7 / 78.1, 227 /
+// 211 (six / two).
 struct TilePlan {
     int ns, w, r;
 };
@@ -468,8 +468,8 @@ int column_cells(bool dp, int m) { return m == 12 ? (dp ? 288 : 368) : m == 8 ? 
 
 // The same for slices the caller chose (lbm_set_variant): the plan's shape where it has as many, else
 // 32 places in FP32, and in FP64 the fewest cells that fill a warp or two evenly (M = 8, two slices,
-// 600^2: 8 places 687 us a step, 8 x 2 354; M = 12, three slices 8 places 1007, 8 x 4 805, six
-// slices 8 places 992, 16 places 759).
+// 600^2: 8 places 693 us a step, 8 x 2 357; M = 12, three slices 8 places 1015, 8 x 4 811, six
+// slices 8 places 1002, 16 places 766).
 TilePlan tile_plan_for(bool dp, int m, long ncells, int ns)
 {
     const TilePlan t = tile_plan(dp, m, ncells);

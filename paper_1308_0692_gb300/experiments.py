@@ -304,7 +304,7 @@ def cavity_hybrid_study(kns=(0.1, 1.0), side=128, n_half=4, layers=(0, 4, 8, 16,
 
 # kernel variants offered to `rates`: (warps per segment, load path); lbm_set_variant rejects
 # the ones without a compiled kernel for a set and precision
-RATE_VARIANTS = [(1, 0), (2, 0), (3, 0), (4, 0), (6, 0), (12, 0), (2, 1), (4, 1), (6, 1), (4, 2), (6, 2),
+RATE_VARIANTS = [(1, 0), (2, 0), (3, 0), (4, 0), (6, 0), (12, 0), (4, 2), (6, 2),
                  (6, 4), (6, 5), (4, 5), (2, 8), (4, 8), (6, 8), (2, 9), (4, 9), (6, 9)]
 
 
